@@ -219,9 +219,11 @@ static void gemm(kf_ctx* c, int kind, int M, int N, int K, const void* A, int ld
     if (!skinny_gemm_supported(g) || launch_gemm_skinny(g, c->d_err, c->stream) != 0) c->launch_failed = true;
   } else if (use_tc) {
     if (launch_gemm_tc(g, c->d_err, c->stream) != 0) c->launch_failed = true;
+  } else if (c->bf16) {
+    launch_gemm_simt(g, c->stream);
+  } else if (launch_gemm_f32(g, c->stream) != 0) {
+    c->launch_failed = true;
   }
-  else
-    launch_gemm_simt(c->bf16, g, c->stream);
   prof_end(c);
 }
 

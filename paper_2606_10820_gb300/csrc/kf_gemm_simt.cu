@@ -1,6 +1,7 @@
-// SIMT GEMM D[M][N] = A[M][K] . W[N][K]^T with fp32 FMA accumulation in
-// ascending k for every output.  Used for the fp32 model (exact-token parity
-// mode) and as the independent GPU check of the tcgen05 GEMM.  A block
+// SIMT GEMM D[M][N] = A[M][K] . W[N][K]^T of bf16 operands with fp32 FMA
+// accumulation in ascending k for every output: the independent GPU check of
+// the tcgen05 GEMM, and the projections of bf16 models whose widths that one
+// does not take (kf_gemm_f32.cu serves the fp32 model).  A block
 // computes 32 rows x 128 columns; warp w owns columns w*32..w*32+31 and lane
 // l owns row l, so each thread ends with one row's run of 32 consecutive
 // columns, the unit the epilogues work on.
@@ -8,8 +9,8 @@
 
 namespace kf {
 
-template <typename TA>
 __global__ void __launch_bounds__(128) k_gemm_simt(GemmDesc g) {
+  using TA = __nv_bfloat16;
   pdl_wait();
   __shared__ float As[32][33];          // [row][k]
   __shared__ __align__(16) float Ws[32][132];  // [k][col]
@@ -52,11 +53,10 @@ __global__ void __launch_bounds__(128) k_gemm_simt(GemmDesc g) {
   if (row < g.M && c0 < g.N) epi_run32<TA>(g.epi, row, c0, acc, g.N);
 }
 
-void launch_gemm_simt(bool bf16, const GemmDesc& g, cudaStream_t s) {
+void launch_gemm_simt(const GemmDesc& g, cudaStream_t s) {
   if (g.M == 0 || g.N == 0) return;
   dim3 grid(ceil_div(g.N, 128), ceil_div(g.M, 32));
-  if (bf16) kf_launch(k_gemm_simt<__nv_bfloat16>, dim3(grid), dim3(128), 0, s, g);
-  else kf_launch(k_gemm_simt<float>, dim3(grid), dim3(128), 0, s, g);
+  kf_launch(k_gemm_simt, dim3(grid), dim3(128), 0, s, g);
 }
 
 }  // namespace kf

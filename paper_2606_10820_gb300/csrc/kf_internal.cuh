@@ -436,8 +436,11 @@ struct GemmDesc {
   size_t l2_bytes = 0;
 };
 
-// SIMT GEMM (any storage type; fp32 accumulation, k ascending per output)
-void launch_gemm_simt(bool bf16, const GemmDesc& g, cudaStream_t s);
+// SIMT GEMM (bf16 operands; fp32 accumulation, k ascending per output)
+void launch_gemm_simt(const GemmDesc& g, cudaStream_t s);
+// the fp32 model's GEMM; -1 if the launch is refused (K, N or a row pitch not
+// a multiple of 4, operands not 16-byte aligned)
+int launch_gemm_f32(const GemmDesc& g, cudaStream_t s);
 
 // tcgen05 GEMM (bf16 only).  Requires K % 64 == 0, 16-byte aligned rows,
 // A rows readable up to round_up(M,128), W rows up to round_up(N,BN).

@@ -111,7 +111,7 @@ extern "C" int kf_op_gemm_bf16(int32_t impl, int32_t M, int32_t N, int32_t K, co
     if (!err) return KF_E_CUDA;
     if (launch_gemm_skinny(g, err, s) != 0) return KF_E_CUDA;
   } else if (impl == KF_GEMM_SIMT) {
-    launch_gemm_simt(true, g, s);
+    launch_gemm_simt(g, s);
   } else {
     return KF_E_ARG;
   }
