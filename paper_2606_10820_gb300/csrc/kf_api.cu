@@ -416,13 +416,14 @@ static void enqueue_step(kf_ctx* c, int B, int P, int k, const float* noise) {
       Epi eh;
       eh.kind = EPI_HEAD; eh.inv_tau = 1.0f / c->cfg.tau; eh.n_valid = c->V;
       eh.rec = c->rec + (size_t)j * B * c->nchunk; eh.nchunk = c->nchunk;
+      eh.want_arg = c->cfg.map_kind == KF_MAP_ARGMAX;
       gemm(c, KF_KIND_GEMM_HEAD, B, c->V_pad, d, c->head_in, d,
            static_cast<const char*>(c->w_mtp) + (size_t)j * c->V_pad * d * c->esz, d, eh);
     }
   } else {
     Epi eh;
     eh.kind = EPI_HEAD; eh.inv_tau = 1.0f / c->cfg.tau; eh.n_valid = c->V; eh.rec = c->rec;
-    eh.nchunk = c->nchunk;
+    eh.nchunk = c->nchunk; eh.want_arg = c->cfg.map_kind == KF_MAP_ARGMAX;
     gemm(c, KF_KIND_GEMM_HEAD, nh, c->V_pad, d, c->head_in, d, c->w_head, d, eh);
   }
   // the noise -> token map, which also commits the step (the emitted tokens

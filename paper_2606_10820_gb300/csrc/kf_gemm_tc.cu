@@ -3,7 +3,8 @@
 //   D[M][N] = A[M][K] . W[N][K]^T, fp32 accumulation in tensor memory.
 //
 // One CTA computes a 128 x BN output tile (MMA M = 128, N = BN, K = 16 per
-// instruction) over a range of 64-wide K blocks.  Warp roles (192 threads):
+// instruction) over a range of 64-wide K blocks (the largest products on CTA
+// pairs: k_gemm_tc_pair).  Warp roles (320 threads):
 //   warp 0      TMA producer: A and W tiles (128B-swizzled, K-major) into a
 //               ring of shared-memory stages, completion on mbarriers;
 //   warp 1      allocates TMEM; one lane issues tcgen05.mma and commits each
@@ -175,6 +176,22 @@ __device__ __forceinline__ void epi_vec_tile(const TcArgs& g, const EpiMeta* met
       bias_lo = __ldg(reinterpret_cast<const float4*>(g.epi.bias + n0 + c + gc));
       if (n0 + c + 32 + gc < g.N) bias_hi = __ldg(reinterpret_cast<const float4*>(g.epi.bias + n0 + c + 32 + gc));
     }
+    if (EPI == EPI_LOGITS) {
+      // the row pitch V need not be a multiple of 4: a row's 32 lanes store
+      // consecutive floats (groups of four per lane wrote quarter sectors)
+      const int rows_w = min(32, g.M - m0 - quarter * 32);
+      const int r_lo = NB >= 2 ? 0 : ch * 16, r_hi = min(rows_w, NB >= 2 ? 32 : ch * 16 + 16);
+      const bool in0 = n0 + c + lane < g.epi.n_valid, in1 = n0 + c + 32 + lane < g.epi.n_valid;
+      float* o = g.epi.outf + (size_t)(m0 + quarter * 32) * g.epi.ldo + n0 + c + lane;
+#pragma unroll 4
+      for (int r = r_lo; r < r_hi; ++r) {
+        const float x = T[r * 68 + lane], y = T[r * 68 + 32 + lane];
+        if (in0) o[(size_t)r * g.epi.ldo] = x * g.epi.inv_tau;
+        if (in1) o[(size_t)r * g.epi.ldo + 32] = y * g.epi.inv_tau;
+      }
+      __syncwarp();
+      continue;
+    }
 #pragma unroll
     for (int ii = 0; ii < NI; ++ii) {
       const int rl = quarter * 32 + gr + 4 * (ibase + ii);   // row within the tile
@@ -218,22 +235,83 @@ __device__ __forceinline__ void epi_vec_tile(const TcArgs& g, const EpiMeta* met
   }
 }
 
+// The LM-head records of one row's 32 logits v / tau for ids col0 .. col0 + 31
+// (those below n_valid): the maximum by three-way maxima in four chains, the
+// sum of 2^((l - m) log2 e) in four packed partial sums (the hardware 2^x,
+// relative error about 2^-22 per term), and, for the argmax map, the lowest
+// id that attains the maximum.  A running argmax and one sum in id order,
+// each a chain of 32 dependent steps, took about 7 us per 128 x 256 tile, twice
+// the tile's mainloop.
+__device__ __forceinline__ void head_record(const Epi& e, int row, int col0, const uint32_t* r) {
+  const int nv = e.n_valid - col0;
+  if (nv <= 0) return;
+  float l[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) l[j] = __uint_as_float(r[j]) * e.inv_tau;
+  if (nv < 32) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) l[j] = j < nv ? l[j] : -INFINITY;
+  }
+  float mq[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int j = 0; j < 32; j += 8)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) mq[c] = max3f(mq[c], l[j + 2 * c], l[j + 2 * c + 1]);
+  HeadRec h;
+  h.m = fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3]));
+  h.a = col0;
+  h.pad = 0;
+  if (e.want_arg) {
+#pragma unroll
+    for (int j = 31; j >= 0; --j) h.a = l[j] == h.m && j < nv ? col0 + j : h.a;
+  }
+  const uint64_t nm = f2(-h.m, -h.m), k2 = f2(1.4426950408889634f, 1.4426950408889634f);
+  uint64_t s[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+  for (int j = 0; j < 32; j += 2) {
+    const float2 x = f2_split(mul_f2(add_f2(f2(l[j], l[j + 1]), nm), k2));
+    float t0, t1;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(x.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(x.y));
+    s[(j >> 1) & 3] = add_f2(s[(j >> 1) & 3], f2(t0, t1));
+  }
+  const float2 t = f2_split(add_f2(add_f2(s[0], s[1]), add_f2(s[2], s[3])));
+  h.s = t.x + t.y;
+  *reinterpret_cast<int4*>(&e.rec[(size_t)row * e.nchunk + col0 / 32]) =
+      make_int4(__float_as_int(h.m), __float_as_int(h.s), h.a, h.pad);
+}
+
+// the records of this thread's row over tile columns [c0, c1) of the
+// accumulator at taddr (warp-collective); the next 32 columns are read from
+// TMEM while this chunk's sum is formed
+__device__ __forceinline__ void head_row(const TcArgs& g, uint32_t taddr, int row, int n0, int c0, int c1) {
+  uint32_t r[2][32];
+  tmem_ld32_async(taddr + c0, r[0]);
+#pragma unroll 1
+  for (int c = c0; c < c1; c += 64) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      tmem_wait32(r[h]);
+      const int cc = c + 32 * h;
+      if (cc + 32 < c1) tmem_ld32_async(taddr + cc + 32, r[h ^ 1]);
+      if (row < g.M && n0 + cc < g.N) head_record(g.epi, row, n0 + cc, r[h]);
+    }
+  }
+}
+
 // ------------------------------------------------------------ the kernel
-// MT: 128-row M tiles per CTA, each with its own TMEM accumulator (2 only for
-// the LM-head records, which need no per-row data); AT: 64-wide K atoms per
-// pipeline stage, so that one mbarrier wait and one commit cover 4 * MT * AT
-// MMAs
-template <int BN, int STAGES, int EPI, int MT, int AT>
+// AT: 64-wide K atoms per pipeline stage, so that one mbarrier wait and one
+// commit cover 4 * AT MMAs
+template <int BN, int STAGES, int EPI, int AT>
 __global__ void __launch_bounds__(kThreads, 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
           TcArgs g) {
   constexpr uint32_t A_ATOM = kBM * kBK * 2;            // one 128 x 64 A box
   constexpr uint32_t B_ATOM = BN * kBK * 2;             // one BN x 64 W box
-  constexpr uint32_t A_BYTES = AT * MT * A_ATOM;        // [atom][M tile] A boxes
-  constexpr uint32_t STAGE_BYTES = AT * (MT * A_ATOM + B_ATOM);   // [A boxes][W atoms]
-  constexpr int TMEM_COLS = tmem_alloc_cols(MT * BN);
-  static_assert(MT * BN <= 512 && BN % 16 == 0 && BN <= 256, "a 128 x BN MMA and its accumulators");
-  static_assert(MT == 1 || EPI == EPI_HEAD, "two M tiles per CTA only for the LM-head records");
+  constexpr uint32_t A_BYTES = AT * A_ATOM;
+  constexpr uint32_t STAGE_BYTES = AT * (A_ATOM + B_ATOM);   // [A boxes][W atoms]
+  constexpr int TMEM_COLS = tmem_alloc_cols(BN);
+  static_assert(BN % 16 == 0 && BN <= 256, "a 128 x BN MMA and its accumulators");
   static_assert(kEpiWarps * 32 * 68 * 4 <= STAGES * STAGE_BYTES &&
                     kBM * (BN + 4) * 4 <= STAGES * STAGE_BYTES,
                 "epilogue blocks and split partials live in the idle pipeline stages");
@@ -249,7 +327,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_tile = blockIdx.x, m_tile = blockIdx.y, split = blockIdx.z;
-  const int n0 = n_tile * BN, m0 = m_tile * kBM * MT;
+  const int n0 = n_tile * BN, m0 = m_tile * kBM;
   const int kb_total = g.K / kBK;
   const int kb0 = split * g.kb_per_split;
   const int kb1 = min(kb_total, kb0 + g.kb_per_split);
@@ -282,12 +360,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
   // warps (idle until the accumulator is ready) each issue their share of a
   // stage's TMA boxes.  One thread issues about one copy per 250 ns whatever
   // its size, so copies from one thread cap the operand stream; warps issue
-  // side by side.  Box j of a stage: K atom j / (MT + 1); A box (M half
-  // j % (MT + 1)) or, for the last one, the W box.  Warp 0 arms each stage's
+  // side by side.  Box j of a stage: K atom j / 2, its A or W box.  Warp 0 arms each stage's
   // barrier.  Weights are constant during a step: the first stages' W boxes
   // stream in while the predecessor kernel finishes; the A boxes it produces
   // are loaded after pdl_wait.
-  constexpr int NBOX = AT * (MT + 1);
+  constexpr int NBOX = 2 * AT;
   constexpr int NPW = NBOX < 4 ? NBOX : 4;
   const int pw = warp == 0 ? 0 : (warp > kThreads / 32 - NPW ? kThreads / 32 - warp : -1);
   if (pw >= 0) {
@@ -308,16 +385,16 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
       // the boxes of stage i that this warp issues: W (w = true) or A boxes
       auto issue = [&](int i, uint32_t sa, uint32_t full, bool w_boxes) {
         const int na = min(AT, nkb - i * AT);
-        for (int j = pw; j < na * (MT + 1); j += NPW) {
-          const int a = j / (MT + 1), r = j % (MT + 1);
+        for (int j = pw; j < na * 2; j += NPW) {
+          const int a = j / 2, r = j % 2;
           const int kc = (kb0 + i * AT + a) * kBK;
-          if (r == MT && w_boxes) tma_load_2d(sa + A_BYTES + a * B_ATOM, &map_w, full, kc, n0);
-          if (r < MT && !w_boxes) tma_load_2d(sa + (a * MT + r) * A_ATOM, &map_a, full, kc, m0 + r * kBM);
+          if (r == 1 && w_boxes) tma_load_2d(sa + A_BYTES + a * B_ATOM, &map_w, full, kc, n0);
+          if (r == 0 && !w_boxes) tma_load_2d(sa + a * A_ATOM, &map_a, full, kc, m0);
         }
       };
       for (int i = 0; i < pre; ++i) {
         const uint32_t full = smem_u32(&bars[i]);
-        if (pw == 0) mbar_expect_tx(full, min(AT, nkb - i * AT) * (MT * g.a_box + B_ATOM));
+        if (pw == 0) mbar_expect_tx(full, min(AT, nkb - i * AT) * (g.a_box + B_ATOM));
         issue(i, smem_u32(smem + i * STAGE_BYTES), full, true);
       }
       pdl_wait();
@@ -327,7 +404,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
         const uint32_t ph = (i / STAGES) & 1;
         if (!mbar_wait(smem_u32(&bars[STAGES + s]), ph ^ 1, g.d_err)) break;
         const uint32_t full = smem_u32(&bars[s]);
-        if (pw == 0) mbar_expect_tx(full, min(AT, nkb - i * AT) * (MT * g.a_box + B_ATOM));
+        if (pw == 0) mbar_expect_tx(full, min(AT, nkb - i * AT) * (g.a_box + B_ATOM));
         const uint32_t sa = smem_u32(smem + s * STAGE_BYTES);
         issue(i, sa, full, true);
         issue(i, sa, full, false);
@@ -354,10 +431,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
           if (a < na) {
 #pragma unroll
             for (int kk = 0; kk < kBK / 16; ++kk)
-#pragma unroll
-              for (int mh = 0; mh < MT; ++mh)
-                mma_bf16(tmem + mh * BN, sdesc(sa + (a * MT + mh) * A_ATOM + kk * 32),
-                         sdesc(sb + a * B_ATOM + kk * 32), idesc, (i > 0 || a > 0 || kk > 0) ? 1u : 0u);
+              mma_bf16(tmem, sdesc(sa + a * A_ATOM + kk * 32), sdesc(sb + a * B_ATOM + kk * 32), idesc,
+                       (i > 0 || a > 0 || kk > 0) ? 1u : 0u);
           }
         }
         mma_commit(smem_u32(&bars[STAGES + s]));
@@ -401,18 +476,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
                 make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         }
       } else if (EPI == EPI_HEAD) {
-        // row mode: a thread reduces its row's 32-id chunks; with two M
-        // tiles the warps of a quarter take one accumulator each, else
-        // alternate halves of the tile's columns
-        const int row = rbase + (MT == 2 ? ch * kBM : 0) + lane;
-        const int c0 = MT == 2 ? 0 : ch * (BN / 2), c1 = MT == 2 ? BN : (ch + 1) * (BN / 2);
-        const uint32_t acc_addr = lane_addr + (MT == 2 ? ch * BN : 0);
-#pragma unroll 1
-        for (int c = c0; c < c1; c += 32) {
-          float v[32];
-          tmem_ld32(acc_addr + c, v);
-          if (row < g.M && n0 + c < g.N) epi_run32<__nv_bfloat16>(g.epi, row, n0 + c, v, g.N);
-        }
+        // row mode: a thread reduces its row's 32-id chunks, the two warps of
+        // a quarter alternate halves of the tile's columns
+        head_row(g, lane_addr, rbase + lane, n0, ch * (BN / 2), (ch + 1) * (BN / 2));
       } else {
         // per epilogue warp a 32 x 68 fp32 block in the idle pipeline stages
         epi_vec_tile<BN, EPI>(g, meta, reinterpret_cast<float*>(smem) + (warp - 2) * (32 * 68), lane_addr, m0, n0,
@@ -696,13 +762,7 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
       if (EPI == EPI_HEAD) {
         // row mode: a thread reduces its row's 32-id chunks, the two warps of
         // a quarter alternate halves of the tile's columns
-        const int r = m0 + quarter * 32 + lane;
-#pragma unroll 1
-        for (int c = ch * (BN / 2); c < (ch + 1) * (BN / 2); c += 32) {
-          float v[32];
-          tmem_ld32(lane_addr + c, v);
-          if (r < g.M && n0 + c < g.N) epi_run32<__nv_bfloat16>(g.epi, r, n0 + c, v, g.N);
-        }
+        head_row(g, lane_addr, m0 + quarter * 32 + lane, n0, ch * (BN / 2), (ch + 1) * (BN / 2));
       } else if (active) {
         epi_vec_tile<BN, EPI>(g, meta, stg + (warp - 2) * (32 * 68), lane_addr, m0, n0, quarter, ch, lane, rows);
       }
@@ -718,6 +778,180 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS)
+                 : "memory");
+}
+
+// ------------------------------------------------------------ CTA pairs
+// The persistent loop over 256 x BN tiles, each computed by the two CTAs of a
+// pair (cta_group::2, M = 256): a CTA stages its 128 rows of A and its half of
+// the W rows, and the tensor cores read the other half from the peer's shared
+// memory.  The leader (rank 0) issues every MMA; both CTAs load their own
+// operands onto the leader's barriers and drain their own 128 rows of the
+// accumulator.  As in the one-CTA loop two TMEM accumulators overlap each
+// tile's epilogue with the next tile's mainloop.
+// Why pairs: shared memory (128 B per clock) bounds the mainloop.  Per 64 of K
+// (512 clocks of MMA at 128 rows x 256 columns per SM) the one-CTA tile writes
+// and reads 48 KB each, 192 B per clock, and measures 0.40 us; a pair's CTA
+// writes and reads 32 KB each, and measures 0.28 us, the tensor cores' rate.
+// Measured, one-CTA loop -> pairs: LM-head records 2048 x 50,257 x 768 119 ->
+// 105 us (with the earlier record epilogue 147); fp32 products 8192 x 4096 x
+// 4096 191 -> 168 us (1.63 PFLOP/s), 4096 x 4096 x 1024 39.0 -> 37.0.
+// With K = 768 and two rounds of tiles the fill (2.4 us) and the last
+// epilogue (4 us) weigh as much as the mainloops, and the projections of a
+// step gain nothing (QKV 26.8 -> 28.4 us at 4096 rows): they stay on the
+// one-CTA kernels.  So do narrower pair tiles (256 x 192 and 256 x 128: slower
+// at every size tried).
+constexpr int kPairThreads = 64 + 32 * kEpiWarps;
+
+template <int BN, int STAGES, int EPI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w, TcArgs g) {
+  constexpr uint32_t A_ATOM = kBM * kBK * 2;
+  constexpr uint32_t B_ATOM = BN / 2 * kBK * 2;
+  constexpr uint32_t STAGE_BYTES = A_ATOM + B_ATOM;
+  constexpr uint32_t STG_BYTES = EPI == EPI_HEAD ? 0 : kEpiWarps * 32 * 68 * 4;
+  constexpr int TMEM_COLS = tmem_alloc_cols(2 * BN);
+  static_assert(EPI == EPI_HEAD || EPI == EPI_LOGITS || EPI == EPI_STORE_F32, "epilogues without per-row data");
+  static_assert(BN % 128 == 0 && BN <= 256 && STAGE_BYTES % 1024 == 0, "half the W rows per CTA, swizzle atoms aligned");
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  float* stg = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES);
+  // full: the leader's, both CTAs' copies of a stage
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES + STG_BYTES);
+  uint64_t* empty = full + STAGES;                          // both: the stage's MMAs are done
+  uint64_t* accf = empty + STAGES;                          // both: accumulator b is complete
+  uint64_t* acce = accf + 2;                                // leader's: the 16 epilogue warps have read b
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const int n_tiles = ceil_div(g.N, BN), m_tiles = ceil_div(g.M, 2 * kBM), tiles = n_tiles * m_tiles;
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+  auto tile_m0 = [&](int t) { return (EPI == EPI_HEAD ? t % m_tiles : t / n_tiles) * 2 * kBM + (int)rank * kBM; };
+  auto tile_n0 = [&](int t) { return (EPI == EPI_HEAD ? t / m_tiles : t % n_tiles) * BN; };
+  const int nkb = g.K / kBK;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < STAGES; ++i) {
+      mbar_init(smem_u32(&full[i]), 1);
+      mbar_init(smem_u32(&empty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&accf[i]), 1);
+      mbar_init(smem_u32(&acce[i]), 2 * kEpiWarps);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_w)) : "memory");
+  }
+  if (warp == 1) {
+    // one warp of each CTA of the pair allocates, collectively
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync();          // both CTAs' barriers are initialised before either is signalled
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      uint32_t stage = 0;
+      bool first = true, live = true;
+      for (int t = pair; live && t < tiles; t += pairs) {
+        const int m0 = tile_m0(t), n0 = tile_n0(t) + (int)rank * (BN / 2);
+        int i0 = 0;
+        if (first) {
+          // weights do not change during a step: the first stages' W boxes
+          // stream in while the predecessor kernel finishes
+          const int pre = min(nkb, STAGES);
+          for (int i = 0; i < pre; ++i) {
+            if (rank == 0) mbar_expect_tx(smem_u32(&full[i]), 2 * STAGE_BYTES);
+            tma_load_2d_pair(smem_u32(smem + i * STAGE_BYTES) + A_ATOM, &map_w, map_rank(smem_u32(&full[i]), 0),
+                             i * kBK, n0);
+          }
+          pdl_wait();
+          for (int i = 0; i < pre; ++i)
+            tma_load_2d_pair(smem_u32(smem + i * STAGE_BYTES), &map_a, map_rank(smem_u32(&full[i]), 0), i * kBK, m0);
+          i0 = pre;
+          first = false;
+        }
+        for (int i = i0; i < nkb; ++i) {
+          const uint32_t sc = stage + i, s = sc % STAGES;
+          if (!mbar_wait_cluster(smem_u32(&empty[s]), ((sc / STAGES) & 1) ^ 1, g.d_err)) {
+            live = false;
+            break;
+          }
+          const uint32_t fb = map_rank(smem_u32(&full[s]), 0);
+          const uint32_t sa = smem_u32(smem + s * STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(smem_u32(&full[s]), 2 * STAGE_BYTES);
+          tma_load_2d_pair(sa, &map_a, fb, i * kBK, m0);
+          tma_load_2d_pair(sa + A_ATOM, &map_w, fb, i * kBK, n0);
+        }
+        stage += nkb;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (rank == 0 && lane == 0) {
+      constexpr uint32_t idesc = idesc_bf16(2 * kBM, BN);
+      uint32_t stage = 0, ti = 0;
+      bool ok = true;   // a timed-out wait ends this pair's tiles
+      for (int t = pair; ok && t < tiles; t += pairs, ++ti) {
+        const uint32_t buf = ti & 1;
+        if (!mbar_wait_cluster(smem_u32(&acce[buf]), ((ti >> 1) & 1) ^ 1, g.d_err)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tmem + buf * BN;
+        for (int i = 0; i < nkb; ++i, ++stage) {
+          const uint32_t s = stage % STAGES;
+          if (!mbar_wait_cluster(smem_u32(&full[s]), (stage / STAGES) & 1, g.d_err)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sa = smem_u32(smem + s * STAGE_BYTES);
+#pragma unroll
+          for (int kk = 0; kk < kBK / 16; ++kk)
+            mma_bf16_pair(d, sdesc(sa + kk * 32), sdesc(sa + A_ATOM + kk * 32), idesc, (i > 0 || kk > 0) ? 1u : 0u);
+          mma_commit_pair(smem_u32(&empty[s]));
+        }
+        if (ok) mma_commit_pair(smem_u32(&accf[buf]));
+      }
+    }
+    __syncwarp();
+  } else {
+    const int quarter = warp & 3;                 // TMEM lanes 32 quarter .. +31
+    const int ch = (warp - 2) >> 2;               // alternate 64-column blocks (records: halves of the tile)
+    pdl_wait();
+    uint32_t ti = 0;
+    for (int t = pair; t < tiles; t += pairs, ++ti) {
+      const uint32_t buf = ti & 1;
+      const int m0 = tile_m0(t), n0 = tile_n0(t);
+      const bool ok = mbar_wait_cluster(smem_u32(&accf[buf]), (ti >> 1) & 1, g.d_err);
+      if (!__all_sync(0xffffffffu, ok)) break;    // timed out: the leader stops too
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t acc = tmem + buf * BN + ((uint32_t)(quarter * 32) << 16);
+      if (EPI == EPI_HEAD) {
+        head_row(g, acc, m0 + quarter * 32 + lane, n0, ch * (BN / 2), (ch + 1) * (BN / 2));
+      } else if (m0 + quarter * 32 < g.M) {
+        EpiRows<BN, EPI> rows;                    // (no per-row data)
+        epi_vec_tile<BN, EPI>(g, nullptr, stg + (warp - 2) * (32 * 68), acc, m0, n0, quarter, ch, lane, rows);
+      }
+      // this warp has read the accumulator: once all 16 have, the leader refills it
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(map_rank(smem_u32(&acce[buf]), 0));
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync();          // no CTA leaves while the other may still signal or read it
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS)
                  : "memory");
 }
 
@@ -801,9 +1035,9 @@ bool tc_gemm_supported(const GemmDesc& g) {
   return get_encode();
 }
 
-template <int BN, int STAGES, int EPI, int MT = 1, int AT = 2>
+template <int BN, int STAGES, int EPI, int AT>
 static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s) {
-  const int n_tiles = ceil_div(g.N, BN), m_tiles = ceil_div(g.M, kBM * MT);
+  const int n_tiles = ceil_div(g.N, BN), m_tiles = ceil_div(g.M, kBM);
   const int tiles = n_tiles * m_tiles;
   const int kb_total = g.K / kBK;
   // split K over a cluster of up to 8 CTAs when the tiles alone leave SMs
@@ -815,9 +1049,9 @@ static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s
     while (splits < 8 && tiles * splits * 2 <= num_sms && kb_total >= splits * 4) splits *= 2;
   int kbps = ceil_div(kb_total, splits);
   splits = ceil_div(kb_total, kbps);   // no empty splits
-  const size_t smem = (size_t)STAGES * AT * (MT * kBM * kBK * 2 + BN * kBK * 2) + 1024 + 256 + sizeof(EpiMeta);
+  const size_t smem = (size_t)STAGES * AT * (kBM * kBK * 2 + BN * kBK * 2) + 1024 + 256 + sizeof(EpiMeta);
   static PerDevice attr, cluster;
-  set_smem_attr(attr, k_gemm_tc<BN, STAGES, EPI, MT, AT>, smem);
+  set_smem_attr(attr, k_gemm_tc<BN, STAGES, EPI, AT>, smem);
   // the largest cluster of these CTAs that fits on one GPC of this device
   const int max_cluster = (int)per_device(cluster, [&] {
     for (int cs = 8; cs > 1; --cs) {
@@ -831,7 +1065,7 @@ static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s
       q.attrs = &ca;
       q.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k_gemm_tc<BN, STAGES, EPI, MT, AT>, &q) == cudaSuccess && n > 0)
+      if (cudaOccupancyMaxActiveClusters(&n, k_gemm_tc<BN, STAGES, EPI, AT>, &q) == cudaSuccess && n > 0)
         return (long long)cs;
       cudaGetLastError();
     }
@@ -845,7 +1079,7 @@ static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s
   // A boxes cover only the rows a tile can hold: at M <= 128 the 128-row MMA
   // reads the rows past the box from stale shared memory, and those rows of
   // the accumulator (all >= M) are never stored
-  const int a_rows = MT == 1 ? std::min(kBM, round_up(g.M, 8)) : kBM;
+  const int a_rows = std::min(kBM, round_up(g.M, 8));
   CUtensorMap ma, mw;
   if (!make_map(&ma, g.A, g.M, g.K, g.lda, a_rows) || !make_map(&mw, g.W, g.N, g.K, g.ldw, BN))
     return -1;
@@ -877,7 +1111,7 @@ static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s
   }
   cfg.attrs = at;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, STAGES, EPI, MT, AT>, ma, mw, a) == cudaSuccess ? 0 : -1;
+  return cudaLaunchKernelEx(&cfg, k_gemm_tc<BN, STAGES, EPI, AT>, ma, mw, a) == cudaSuccess ? 0 : -1;
 }
 
 template <int BN, int STAGES, int EPI>
@@ -923,39 +1157,82 @@ static int launch_persist(const GemmDesc& g, int* d_err, int num_sms, cudaStream
   return -1;
 }
 
+template <int BN, int STAGES, int EPI>
+static int launch_pair_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s) {
+  const int tiles = ceil_div(g.N, BN) * ceil_div(g.M, 2 * kBM);
+  const size_t smem = (size_t)STAGES * (kBM * kBK * 2 + BN / 2 * kBK * 2) +
+                      (EPI == EPI_HEAD ? 0 : kEpiWarps * 32 * 68 * 4) + 1024 + 256;
+  static PerDevice attr;
+  set_smem_attr(attr, k_gemm_tc_pair<BN, STAGES, EPI>, smem);
+  CUtensorMap ma, mw;
+  if (!make_map(&ma, g.A, g.M, g.K, g.lda, kBM) || !make_map(&mw, g.W, g.N, g.K, g.ldw, BN / 2)) return -1;
+  TcArgs a;
+  a.M = g.M; a.N = g.N; a.K = g.K; a.kb_per_split = g.K / kBK; a.splits = 1;
+  a.a_box = 0;
+  a.l2_next = nullptr; a.l2_bytes = 0;
+  a.d_err = d_err; a.epi = g.epi;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * std::min(tiles, num_sms / 2));
+  cfg.blockDim = dim3(kPairThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = g_pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_gemm_tc_pair<BN, STAGES, EPI>, ma, mw, a) == cudaSuccess ? 0 : -1;
+}
+
 template <int BN, int STAGES, int AT>
 static int launch_bn(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s) {
   switch (g.epi.kind) {
-    case EPI_STORE: return launch_epi<BN, STAGES, EPI_STORE, 1, AT>(g, d_err, num_sms, s);
-    case EPI_BIAS_GELU: return launch_epi<BN, STAGES, EPI_BIAS_GELU, 1, AT>(g, d_err, num_sms, s);
-    case EPI_RESID: return launch_epi<BN, STAGES, EPI_RESID, 1, AT>(g, d_err, num_sms, s);
-    case EPI_NOISE_OUT: return launch_epi<BN, STAGES, EPI_NOISE_OUT, 1, AT>(g, d_err, num_sms, s);
-    case EPI_LOGITS: return launch_epi<BN, STAGES, EPI_LOGITS, 1, AT>(g, d_err, num_sms, s);
-    case EPI_STORE_F32: return launch_epi<BN, STAGES, EPI_STORE_F32, 1, AT>(g, d_err, num_sms, s);
-    case EPI_QKV: return launch_epi<BN, STAGES, EPI_QKV, 1, AT>(g, d_err, num_sms, s);
+    case EPI_STORE: return launch_epi<BN, STAGES, EPI_STORE, AT>(g, d_err, num_sms, s);
+    case EPI_BIAS_GELU: return launch_epi<BN, STAGES, EPI_BIAS_GELU, AT>(g, d_err, num_sms, s);
+    case EPI_RESID: return launch_epi<BN, STAGES, EPI_RESID, AT>(g, d_err, num_sms, s);
+    case EPI_NOISE_OUT: return launch_epi<BN, STAGES, EPI_NOISE_OUT, AT>(g, d_err, num_sms, s);
+    case EPI_LOGITS: return launch_epi<BN, STAGES, EPI_LOGITS, AT>(g, d_err, num_sms, s);
+    case EPI_STORE_F32: return launch_epi<BN, STAGES, EPI_STORE_F32, AT>(g, d_err, num_sms, s);
+    case EPI_QKV: return launch_epi<BN, STAGES, EPI_QKV, AT>(g, d_err, num_sms, s);
   }
   return -1;
 }
 
 int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   const int num_sms = device_sms();
-  // LM-head records: 256-wide tiles; above 128 rows both M tiles of a row
-  // pair in one CTA (each weight tile is streamed from HBM once per 256 rows)
+  const bool persist = !(g_gemm_flags & kGemmNoPersist);
+  // CTA pairs where their rounds of 256 x 256 tiles are many and deep enough
+  // to outweigh the pair's start (about 4 us) and its coarser rounds; one-CTA
+  // loop -> pairs, microseconds: records 2048 x 50,257 at K = 1024 162 -> 146,
+  // K = 768 147 -> 134, 1024 x 50,257 x 768 (11 rounds) 74.3 -> 71.5, 512 x
+  // 50,257 x 1024 (6) 57.3 -> 52.7; but 1024 x 30,522 x 768 (7) 47.6 -> 51.5,
+  // 2100 x 50,257 x 256 82 -> 99; logits 2048 x 50,257 197 -> 179; fp32
+  // products 4096 x 4096 x 1024 (4) 39.0 -> 37.0, 4096 x 3072 x 768 (3) 25.3 -> 26.0
+  const long long depth = (long long)ceil_div(ceil_div(g.N, 256) * ceil_div(g.M, 2 * kBM), num_sms / 2) * g.K;
+  if (persist && ceil_div(g.N, 256) * ceil_div(g.M, kBM) > num_sms && num_sms >= 2 &&   // (no split-K below either)
+      (depth >= 6144 || (g.K >= 1024 && depth >= 4096))) {
+    if (g.epi.kind == EPI_HEAD) return launch_pair_epi<256, 6, EPI_HEAD>(g, d_err, num_sms, s);
+    if (g.epi.kind == EPI_LOGITS) return launch_pair_epi<256, 4, EPI_LOGITS>(g, d_err, num_sms, s);
+    if (g.epi.kind == EPI_STORE_F32) return launch_pair_epi<256, 4, EPI_STORE_F32>(g, d_err, num_sms, s);
+  }
+  // LM-head records: 256-wide tiles
   if (g.epi.kind == EPI_HEAD) {
     // above one M tile, more than a wave of 128 x 256 tiles: a persistent
     // loop, the M tiles of each weight tile side by side (the weights are read
     // from HBM once) and each tile's records overlapping the next tile's
     // mainloop
-    if (g.M > kBM && !(g_gemm_flags & kGemmNoPersist) && ceil_div(g.N, 256) * ceil_div(g.M, kBM) > num_sms)
+    if (g.M > kBM && persist && ceil_div(g.N, 256) * ceil_div(g.M, kBM) > num_sms)
       return launch_persist<256, 3>(g, d_err, num_sms, s);
-    if (g.M > kBM) return launch_epi<256, 3, EPI_HEAD, 2, 1>(g, d_err, num_sms, s);
     // one M tile, more than a wave of 256-wide tiles (the OWT-shaped vocab:
     // 197 tiles on 152 SMs left a second wave of 45): a persistent loop over
     // 128-wide tiles keeps every SM streaming weights to the end (batch 1,
     // k = 4: 309.5 -> 303.8 us per call)
-    if (!(g_gemm_flags & kGemmNoPersist) && ceil_div(g.N, 256) > num_sms)
+    if (g.M <= kBM && persist && ceil_div(g.N, 256) > num_sms)
       return launch_persist_epi<128, 4, EPI_HEAD>(g, d_err, num_sms, s);
-    return launch_epi<256, 2, EPI_HEAD, 1, 2>(g, d_err, num_sms, s);
+    // within a wave a CTA per 128 x 256 tile (two M tiles per CTA, which
+    // stream a weight tile once, left SMs idle: 2048 rows x 1000 ids x 1024
+    // 27.5 us)
+    return launch_epi<256, 2, EPI_HEAD, 2>(g, d_err, num_sms, s);
   }
   // the narrowest tile that covers the product in one wave, else 256-wide
   // tiles: a tcgen05.mma re-reads its whole 128-row A operand from shared

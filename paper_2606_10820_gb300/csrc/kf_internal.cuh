@@ -142,6 +142,7 @@ struct Epi {
   int n_valid = 0;
   HeadRec* rec = nullptr;
   int nchunk = 0;
+  bool want_arg = true;         // EPI_HEAD: the argmax map reads the records' ids
   // EPI_QKV
   float* q_out = nullptr;          // [rows][H][64]
   void* kv = nullptr;              // [L][n_pages][2][H][16][64]

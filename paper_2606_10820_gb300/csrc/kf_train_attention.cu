@@ -406,33 +406,6 @@ __device__ __forceinline__ void pair_bar(int quarter) {
   asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
 }
 
-// three-way max, and packed pairs of fp32 (two lanes of one 64-bit register)
-__device__ __forceinline__ float max3f(float x, float y, float z) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(x), "f"(y), "f"(z));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2(float x, float y) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ float2 f2_split(uint64_t p) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma_f2(uint64_t x, uint64_t y, uint64_t z) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
-  return r;
-}
-__device__ __forceinline__ uint64_t add_f2(uint64_t x, uint64_t y) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
-  return r;
-}
-
 // first key and range end of tile j of an item (constant indices only: the
 // ranges stay in registers)
 __device__ __forceinline__ void tile_at(const TileRanges& r, int j, int* lo, int* hi) {

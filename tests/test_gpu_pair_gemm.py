@@ -1,0 +1,55 @@
+"""Products on CTA pairs (256 x 256 tiles, both CTAs' operands and
+accumulators) and the LM-head records' reductions, at their edges, against
+fp64 matmuls (needs a GB300)."""
+import numpy as np
+import pytest
+
+from test_gpu_gemm import _run
+from test_gpu_gemm import env  # noqa: F401
+from test_gpu_head_op import _case, check_against_oracle, run_op
+from test_gpu_head_op import env as head_env  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (2100, 2340, 3072),     # ragged in both; the second CTA's last tile is empty (rows 2100 .. past 2176)
+    (4500, 1028, 4096),     # 20 rows in the last pair's second CTA, 4 columns in the last tile
+    (19500, 64, 3072),      # one narrow column tile, 77 pairs of row tiles on 76 CTA pairs
+    (4096, 4096, 1024),     # full tiles, four rounds
+])
+def test_pair_gemm_matches_fp64_matmul(env, M, N, K):  # noqa: F811
+    torch, lib = env
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = (torch.randn(M, K, device="cuda", generator=g) * 0.5).to(torch.bfloat16)
+    W = (torch.randn(N, K, device="cuda", generator=g) * 0.02).to(torch.bfloat16)
+    ref = A.double() @ W.double().T
+    out = _run(torch, lib, 0, A, W)
+    # products are exact in fp32; the tensor cores' K-long fp32 accumulation
+    # measures 1.1e-9 K relative to the result: four times that
+    rel = ((out.double() - ref).norm() / ref.norm()).item()
+    assert rel <= 4.4e-9 * K + 1e-7
+    # each 128 x 256 tile sees the K order of a CTA per tile: identical bits
+    assert torch.equal(out, _run(torch, lib, 2, A, W))
+
+
+# (400 x 25,000 x 3072: the records on CTA pairs, a ragged second row pair;
+# vocabularies that end inside a chunk, at one id, on a chunk; fewer than a
+# wave of row tiles; argmax ties within and across chunks below)
+@pytest.mark.parametrize("rows,V,d", [(400, 25000, 3072), (129, 33, 64), (7, 1, 64), (300, 992, 128), (2048, 1000, 128)])
+@pytest.mark.parametrize("map_kind", [0, 1])
+def test_head_records_at_edges(head_env, rows, V, d, map_kind):  # noqa: F811
+    torch, lib = head_env
+    x, w, z = _case(torch, rows, V, d, rows + V)
+    got = run_op(lib, torch, x, w, z, 1.0, map_kind)
+    assert check_against_oracle(x, w, z, 1.0, map_kind, got) == 0
+
+
+@pytest.mark.parametrize("ids", [(5, 9), (31, 32), (40, 95), (64, 998)])
+def test_argmax_ties_take_the_lowest_id(head_env, ids):  # noqa: F811
+    torch, lib = head_env
+    x, w, z = _case(torch, 130, 1000, 64, 3)
+    w[list(ids)] = (x[0].float() * 0.5).to(torch.bfloat16)
+    got = run_op(lib, torch, x, w, z, 1.0, 1)
+    lg = (x[0].double() @ w.double().T).cpu().numpy()
+    assert np.argmax(lg) == ids[0] and got[0] == ids[0]
