@@ -27,8 +27,11 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <utility>
+#include <vector>
 
 #include "../../include/kforcing_ops.h"
+#include "kf_attn_tc.cuh"
 #include "kf_internal.cuh"
 #include "kf_mma.cuh"
 #include "kf_tc.cuh"
@@ -50,10 +53,7 @@ struct TrainAttnArgs {
   int N, kw, blocks, T, H, q_begin, q_end, dense;
 };
 
-// the keys row qi sees: context keys <= ctx, and [w1lo, w1hi), [w2lo, w2hi)
-struct RowVis {
-  int ctx, w1lo, w1hi, w2lo, w2hi;
-};
+using fa::RowVis;
 
 __device__ __forceinline__ RowVis row_vis(const TrainAttnArgs& a, int qi) {
   RowVis r{-1, 0, 0, 0, 0};
@@ -288,489 +288,104 @@ __global__ void __launch_bounds__(kThr, 3) k_train_attention(TrainAttnArgs a) {
 }
 
 // ------------------------------------------------------------------ tcgen05
-// The same attention on the 5th-generation tensor cores.  A work item is 128
-// query rows of one (sequence, head); its key ranges are walked in tiles of
-// 128 keys (each range's tiles start at its first key; keys past the range's
-// end are masked, so no key is counted twice).  The kernel is persistent:
-// one CTA per SM takes items blockIdx.x, blockIdx.x + gridDim.x, ... (the
-// query tiles with the most keys first), and its roles run ahead across
-// items, so that the next item's copies and first products overlap this
-// item's last softmax tile and output:
-//   warp 0      TMA: an item's Q (once the previous item's last S product
-//               has read the Q buffer), then its K and V tiles of
-//               [128 keys][64] bf16 (128-byte swizzle) into a four-stage ring;
-//   warp 1      one thread issues tcgen05.mma: S_j = Q K_j^T (M = 128 rows,
-//               N = 128 keys, K = 64) into one of two TMEM buffers, and
-//               O += P_j V_j (M = 128, N = 64, K = 128 keys; V is the
-//               MN-major operand as loaded) into one TMEM accumulator, an
-//               item's first P V overwriting it once the softmax has read
-//               the previous item's O;
-//   warps 2..9  two threads per query row (TMEM lane), each with half of
-//               its keys and of its output (four threads measured 5 % slower:
-//               the per-tile chain of waits and barriers, not the arithmetic,
-//               bounds the softmax): mask S_j, share the row max with the
-//               partner warp (the other half of the same rows) through shared
-//               memory and a barrier of the pair, keep a reference max m and
-//               their part of the sum l, and write P_j = exp2(S_j - m) as
-//               bf16 into shared memory (K-major, swizzled: the A operand of
-//               P V); every softmax thread arrives on the barrier that
-//               releases P_j to the tensor cores.  m
-//               is raised only when a tile's max exceeds it by more than 2^8
-//               (P stays below 256); then O in TMEM and l are scaled to the
-//               new m before P_j is released.  At the item's end O / l is
-//               the row's output.
-// Tiles are numbered across the CTA's items (g): S of tile g + 1 is computed
-// while the softmax works on tile g, and P V of tile g is issued after it
-// (an item's last P V right after its last S).
-// Every wait is bounded; a wait that runs out sets the error word and ends
-// the CTA's loops.
+// The same attention on the 5th-generation tensor cores (k_attn_tc): an item is
+// up to 128 query rows of one (sequence, head), all of the context or of one
+// block.  A block's tiles hold whole windows (floor(128 / k) k rows, anchored
+// at the block's start), so that their keys in each block fit one 128-key
+// tile; tiles cut at 128 rows opened up to two tiles per block, and a tile
+// across two parts of the layout the ranges of both.
 namespace {
-constexpr int kTcRows = 128;
-constexpr int kTcKeys = 128;
-constexpr int kTcSplit = 2;                          // softmax threads per query row
-constexpr int kTcSoftmax = 128 * kTcSplit;           // kTcSplit warps per TMEM lane quarter
-constexpr int kTcThreads = 64 + kTcSoftmax;
-constexpr int kTcPart = kTcKeys / kTcSplit;          // keys of a row per softmax thread
-constexpr int kTcOut = kHD / kTcSplit;               // output dims of a row per softmax thread
-constexpr uint32_t kTcTile = kTcRows * kHD * 2;       // 16 KB: Q, a K tile, a V tile
-constexpr uint32_t kTcP = kTcRows * kTcKeys * 2;      // 32 KB: one P tile (two 64-key atoms)
-// K/V ring stages: tile j's copies are issued while tile j - 1 is in the
-// softmax and tile j - 2's V still feeds P V (two stages measured 2.0 us per
-// tile, the copy latency on the critical path)
-constexpr int kTcStages = 4;
-// [Q][K stages][V stages][P 2], the barriers and shared scalars (256 B),
-// then the row-max exchange [2 tiles][kTcSplit parts][128 rows] and the row
-// sums [2 items][kTcSplit][128]
-constexpr size_t tc_smem_bytes() {
-  return 1024 + (1 + 2 * kTcStages) * (size_t)kTcTile + 2 * (size_t)kTcP + 256 + 4 * kTcSplit * 128 * 4;
-}
-
-// The key ranges an item's 128 query rows open (the union over its rows:
-// the context prefix up to the largest context key, the block-1 and block-2
-// windows; an empty one has lo == hi), the smallest context key every valid
-// row sees, and the number of 128-key tiles.  Warp-collective: each lane
-// takes four rows.
-struct TileRanges {
-  int lo[3], hi[3], cmin, n;
+constexpr int kTileList = 448;
+struct TrainArgs {
+  TrainAttnArgs a;
+  int n_batch, qr;                       // qr: rows of a block's query tile
+  int first[3], count[3];                // query tiles of the context (0) and the blocks (1, 2)
+  int n_qt;
+  int q0[kTileList];                     // their first rows, most keys first (n_qt <= kTileList)
 };
+struct TrainPolicy {
+  using Args = TrainArgs;
+  struct Maps { CUtensorMap q, k, v; };
+  struct Item { int q0, q1, h, b; };     // rows q0 .. q1 - 1 (at most 128)
+  struct TileRef { int kt; };
+  static constexpr bool kQByRows = false, kZeroV = false, kWindows = true;
 
-__device__ __forceinline__ TileRanges tile_ranges(const TrainAttnArgs& a, int q0, int lane) {
-  int cmax = -1, cmin = 1 << 30, w1lo = 1 << 30, w1hi = 0, w2lo = 1 << 30, w2hi = 0;
-#pragma unroll
-  for (int i = 0; i < kTcRows / 32; ++i) {
-    const RowVis v = row_vis(a, q0 + lane + 32 * i);
-    if (v.ctx < 0) continue;
-    cmax = max(cmax, v.ctx);
-    cmin = min(cmin, v.ctx);
-    if (v.w1hi > v.w1lo) { w1lo = min(w1lo, v.w1lo); w1hi = max(w1hi, v.w1hi); }
-    if (v.w2hi > v.w2lo) { w2lo = min(w2lo, v.w2lo); w2hi = max(w2hi, v.w2hi); }
-  }
-  cmax = __reduce_max_sync(0xffffffffu, cmax);
-  cmin = __reduce_min_sync(0xffffffffu, cmin);
-  w1lo = __reduce_min_sync(0xffffffffu, w1lo);
-  w1hi = __reduce_max_sync(0xffffffffu, w1hi);
-  w2lo = __reduce_min_sync(0xffffffffu, w2lo);
-  w2hi = __reduce_max_sync(0xffffffffu, w2hi);
-  TileRanges r;
-  if (a.dense) {
-    r.lo[0] = 0; r.hi[0] = a.T;
-    r.lo[1] = r.hi[1] = r.lo[2] = r.hi[2] = 0;
-  } else {
-    r.lo[0] = 0; r.hi[0] = cmax + 1;                              // 0 when no valid row
-    r.lo[1] = w1lo; r.hi[1] = max(w1lo, w1hi);
-    r.lo[2] = w2lo; r.hi[2] = max(w2lo, w2hi);
-  }
-  r.cmin = cmin;
-  r.n = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) r.n += ceil_div(r.hi[i] - r.lo[i], kTcKeys);
-  return r;
-}
+  static __device__ __forceinline__ int n_items(const Args& g) { return g.n_qt * g.a.H * g.n_batch; }
+  static __device__ __forceinline__ bool all_open(const Args& g) { return !g.a.dense; }
 
-// The two softmax warps of a TMEM lane quarter hold the two parts of the same
-// rows; they meet on named barrier 2 + quarter (64 threads), which also ORs
-// a predicate over them: both get the same answer and leave a loop together.
-__device__ __forceinline__ bool pair_bar_or(int quarter, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.or.pred q, %2, 64, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)pred), "r"(2 + quarter)
-      : "memory");
-  return r != 0;
-}
-__device__ __forceinline__ void pair_bar(int quarter) {
-  asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
-}
-
-// first key and range end of tile j of an item (constant indices only: the
-// ranges stay in registers)
-__device__ __forceinline__ void tile_at(const TileRanges& r, int j, int* lo, int* hi) {
-  *lo = 0; *hi = 0;
+  // Item w: query tile rank w / (H B), most keys first, then head and
+  // sequence.  The host lists the tiles' first rows (working a tile out of its
+  // rank in the kernel took a tenth of its instructions); past kTileList tiles
+  // each part of the layout is walked from its end, the blocks first.
+  static __device__ __forceinline__ void item(const Args& g, int w, int lane, Item& im, fa::Ranges& r) {
+    const TrainAttnArgs& a = g.a;
+    const int n_hb = a.H * g.n_batch, rank = w / n_hb, hb = w - rank * n_hb;
+    im.b = hb / a.H;
+    im.h = hb - im.b * a.H;
+    const int Nk = a.N * a.kw;
+    if (g.n_qt <= kTileList) {
+      im.q0 = g.q0[rank];
+    } else if (rank < g.count[2]) {
+      im.q0 = a.N + Nk + (g.first[2] + g.count[2] - 1 - rank) * g.qr;
+    } else if (rank < g.count[2] + g.count[1]) {
+      im.q0 = a.N + (g.first[1] + g.count[1] + g.count[2] - 1 - rank) * g.qr;
+    } else {
+      im.q0 = (g.first[0] + g.n_qt - 1 - rank) * fa::kRows;
+    }
+    const int part = im.q0 < a.N ? 0 : im.q0 < a.N + Nk ? 1 : 2;
+    const int bs = part == 0 ? 0 : a.N + (part - 1) * Nk;
+    const int len = part == 0 ? a.N : Nk, rows = part == 0 ? fa::kRows : g.qr;
+    im.q1 = min(min(im.q0 + rows, bs + len), a.q_end);
+    const int lo = max(im.q0, a.q_begin), hi = im.q1 - 1;   // the item's valid rows
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const int n = ceil_div(r.hi[i] - r.lo[i], kTcKeys);
-    if (j >= 0 && j < n) { *lo = r.lo[i] + j * kTcKeys; *hi = r.hi[i]; }
-    j -= n;
+    for (int x = 0; x < 3; ++x) r.lo[x] = r.hi[x] = 0;
+    if (part == 0) {
+      r.cmin = lo;
+      r.hi[0] = hi + 1;
+    } else {
+      const int t0 = (lo - bs) / a.kw, t1 = (hi - bs) / a.kw;
+      r.cmin = t0;
+      r.hi[0] = t1 + 1;
+      r.lo[1] = a.N + t0 * a.kw;
+      r.hi[1] = part == 1 ? hi + 1 : a.N + (t1 + 1) * a.kw;
+      if (part == 2) {
+        r.lo[2] = bs + t0 * a.kw;
+        r.hi[2] = hi + 1;
+      }
+    }
+    if (a.dense) {
+#pragma unroll
+      for (int x = 0; x < 3; ++x) r.lo[x] = r.hi[x] = 0;
+      r.hi[0] = a.T;
+    }
+    fa::count_tiles(r);
   }
-}
+  static __device__ __forceinline__ RowVis vis(const Args& g, const Item& im, int row) {
+    return im.q0 + row < im.q1 ? row_vis(g.a, im.q0 + row) : RowVis{-1, 0, 0, 0, 0};
+  }
+  static __device__ __forceinline__ void load_q(const Maps& m, const Item& im, uint32_t dst, uint32_t bar) {
+    tma_load_4d(dst, &m.q, bar, 0, im.h, im.q0, im.b);
+  }
+  static __device__ __forceinline__ void q_rows(const Args&, const Item&, uint8_t*, int, int) {}
+  static __device__ __forceinline__ TileRef tile(const Args&, const Item&, int kt, int, int, int*) { return {kt}; }
+  static __device__ __forceinline__ uint32_t tile_bytes(const TileRef&) { return fa::kTileBytes; }   // (rows past T: zeros)
+  static __device__ __forceinline__ void load_k(const Maps& m, const Args&, const Item& im, const TileRef& r, int lane,
+                                                uint32_t dst, uint32_t bar) {
+    if (lane == 0) tma_load_4d(dst, &m.k, bar, 0, im.h, r.kt, im.b);
+  }
+  static __device__ __forceinline__ void load_v(const Maps& m, const Args&, const Item& im, const TileRef& r, int lane,
+                                                uint32_t dst, uint32_t bar) {
+    if (lane == 0) tma_load_4d(dst, &m.v, bar, 0, im.h, r.kt, im.b);
+  }
+  static __device__ __forceinline__ void store(const Args& g, const Item& im, int row, const float* o, float inv) {
+    const TrainAttnArgs& a = g.a;
+    float* dst = a.out + (((size_t)im.b * (a.q_end - a.q_begin) + (im.q0 + row - a.q_begin)) * a.H + im.h) * kHD;
+#pragma unroll
+    for (int d = 0; d < kHD; d += 4)
+      *reinterpret_cast<float4*>(dst + d) = make_float4(o[d] * inv, o[d + 1] * inv, o[d + 2] * inv, o[d + 3] * inv);
+  }
+};
 }  // namespace
-
-__global__ void __launch_bounds__(kTcThreads, 1)
-k_train_attention_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                     const __grid_constant__ CUtensorMap map_v, TrainAttnArgs a, int n_batch, int* d_err) {
-  extern __shared__ __align__(1024) uint8_t tsm_raw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tsm_raw) + 1023) & ~uintptr_t(1023));
-  const uint32_t sQ = smem_u32(sm);
-  const uint32_t sK = sQ + kTcTile;                  // [kTcStages]
-  const uint32_t sV = sK + kTcStages * kTcTile;      // [kTcStages]
-  constexpr uint32_t kPOff = (1 + 2 * kTcStages) * kTcTile;
-  uint8_t* Pp = sm + kPOff;                          // [2][2 atoms][128 rows][128 B]
-  const uint32_t sP = smem_u32(Pp);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kPOff + 2 * kTcP);
-  uint64_t* q_full = bars;
-  uint64_t* q_empty = bars + 1;                      // the item's last S product done
-  uint64_t* kv_full = bars + 2;                      // [kTcStages]
-  uint64_t* kv_empty = kv_full + kTcStages;          // [kTcStages]
-  uint64_t* s_full = kv_empty + kTcStages;           // [2]
-  uint64_t* p_full = s_full + 2;                     // [2]: P_g written (and S_g read)
-  uint64_t* o_full = p_full + 2;                     // [2]
-  uint64_t* o_free = o_full + 2;                     // the item's O read out
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 1);
-  int* s_cnt = reinterpret_cast<int*>(tmem_slot + 1);    // K/V tiles the MMA thread has taken
-  int* s_qcnt = s_cnt + 1;                               // Q tiles the MMA thread has taken
-  float* s_mx = reinterpret_cast<float*>(sm + kPOff + 2 * kTcP + 256);         // [2][kTcSplit][128]
-  float* s_l = s_mx + 2 * kTcSplit * kTcRows;                                  // [2][kTcSplit][128]
-
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const int quarter = warp & 3;                 // softmax warps: TMEM lanes 32 quarter ..
-  const int row = 32 * quarter + lane;          // this softmax thread's query row in the tile
-  const int part = (warp - 2) >> 2;             // its keys kTcPart part .. and output dims kTcOut part ..
-  const int n_qt = ceil_div(a.q_end - a.q_begin, kTcRows);
-  const int n_hb = a.H * n_batch;
-  const int n_items = n_qt * n_hb;
-  // the CTA's i-th item: rounds of gridDim.x items, walked forwards in even
-  // rounds and backwards in odd ones, so that each CTA's items add up to
-  // about the same number of tiles; -1 past the last
-  auto item_at = [&](int i) -> int {
-    const int P = gridDim.x, c = blockIdx.x;
-    const long long w = (long long)i * P + ((i & 1) ? P - 1 - c : c);
-    return w < n_items ? (int)w : -1;
-  };
-  // item w: query tile n_qt - 1 - w / n_hb (the most keys first), then head
-  // and sequence
-  auto item = [&](int w, int* q0, int* h, int* b) {
-    const int qt = w / n_hb, hb = w - qt * n_hb;
-    *q0 = a.q_begin + (n_qt - 1 - qt) * kTcRows;
-    *h = hb % a.H;
-    *b = hb / a.H;
-  };
-
-  if (t == 0) {
-    mbar_init(smem_u32(q_full), 1);
-    mbar_init(smem_u32(q_empty), 1);
-    for (int i = 0; i < kTcStages; ++i) {
-      mbar_init(smem_u32(&kv_full[i]), 1);
-      mbar_init(smem_u32(&kv_empty[i]), 1);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&s_full[i]), 1);
-      mbar_init(smem_u32(&p_full[i]), kTcSoftmax);      // every softmax thread
-      mbar_init(smem_u32(&o_full[i]), 1);
-    }
-    mbar_init(smem_u32(o_free), kTcSoftmax);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_q)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_k)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_v)) : "memory");
-    s_cnt[0] = 0;
-    s_qcnt[0] = 0;
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(512)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
-  pdl_wait();
-
-  if (warp == 0) {
-    bool ok = true;
-    int g = 0, issued = 0, q_issued = 0, it = 0;
-    for (int w = item_at(0); ok && w >= 0; w = item_at(++it)) {
-      int q0, h, b;
-      item(w, &q0, &h, &b);
-      const TileRanges r = tile_ranges(a, q0, lane);
-      if (lane == 0) {
-        // the Q buffer is free once the previous item's last S product is done
-        if (it > 0 && !mbar_wait(smem_u32(q_empty), (it - 1) & 1, d_err)) ok = false;
-        if (ok) {
-          mbar_expect_tx(smem_u32(q_full), kTcTile);
-          tma_load_4d(sQ, &map_q, smem_u32(q_full), 0, h, q0, b);
-          q_issued = it + 1;
-        }
-        for (int j = 0; ok && j < r.n; ++j, ++g) {
-          const int st = g % kTcStages;
-          if (g >= kTcStages && !mbar_wait(smem_u32(&kv_empty[st]), ((g / kTcStages) - 1) & 1, d_err)) {
-            ok = false;
-            break;
-          }
-          int kt, kend;
-          tile_at(r, j, &kt, &kend);
-          mbar_expect_tx(smem_u32(&kv_full[st]), 2 * kTcTile);
-          tma_load_4d(sK + st * kTcTile, &map_k, smem_u32(&kv_full[st]), 0, h, kt, b);
-          tma_load_4d(sV + st * kTcTile, &map_v, smem_u32(&kv_full[st]), 0, h, kt, b);
-          issued = g + 1;
-        }
-      }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-    }
-    if (lane == 0 && !ok) {
-      // let the copies still in flight land before the CTA ends (bounded)
-      for (int j = *(volatile int*)s_cnt; j < issued; ++j)
-        mbar_wait(smem_u32(&kv_full[j % kTcStages]), (j / kTcStages) & 1, d_err);
-      if (q_issued > *(volatile int*)s_qcnt) mbar_wait(smem_u32(q_full), (q_issued - 1) & 1, d_err);
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    constexpr uint32_t idesc_s = idesc_bf16(kTcRows, kTcKeys);
-    constexpr uint32_t idesc_o = idesc_bf16(kTcRows, kHD) | (1u << 16);   // B (V) MN-major
-    bool ok = true;
-    int g = 0, it = 0, o_items = 0;
-    int pv = -1;                  // the tile whose S is issued and whose P V is not
-    bool pv_first = false;        // ... the first tile of its item
-    // O += P_i V_i in TMEM columns 256 .. 319.  An item's first tile
-    // overwrites O once the softmax has read the previous item's O out; the
-    // softmax rescales O in place before it releases P_i when the row max
-    // has grown.
-    auto issue_pv = [&](int i, bool first) -> bool {
-      if (first) {
-        if (o_items > 0 && !mbar_wait(smem_u32(o_free), (o_items - 1) & 1, d_err)) return false;
-        ++o_items;
-      }
-      const int st = i & 1;
-      if (!mbar_wait(smem_u32(&p_full[st]), (i >> 1) & 1, d_err)) return false;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int kvs = i % kTcStages;
-      const uint32_t pa = sP + st * kTcP, vb = sV + kvs * kTcTile;
-#pragma unroll
-      for (int kk = 0; kk < kTcKeys / 16; ++kk)
-        mma_bf16(tmem + 256, sdesc(pa + (kk >> 2) * (kTcP / 2) + (kk & 3) * 32),
-                 sdesc_mn(vb + kk * 16 * 128), idesc_o, (!first || kk > 0) ? 1u : 0u);
-      mma_commit(smem_u32(&o_full[st]));
-      mma_commit(smem_u32(&kv_empty[kvs]));
-      return true;
-    };
-    for (int w = item_at(0); ok && w >= 0; w = item_at(++it)) {
-      int q0, h, b;
-      item(w, &q0, &h, &b);
-      const TileRanges r = tile_ranges(a, q0, lane);
-      if (lane == 0) {
-        ok = mbar_wait(smem_u32(q_full), it & 1, d_err);
-        if (ok) *(volatile int*)s_qcnt = it + 1;
-        for (int j = 0; ok && j < r.n; ++j, ++g) {
-          const int st = g & 1;
-          if (!mbar_wait(smem_u32(&kv_full[g % kTcStages]), (g / kTcStages) & 1, d_err)) { ok = false; break; }
-          *(volatile int*)s_cnt = g + 1;
-          // S buffer st is free once the softmax has read S_{g-2}
-          if (g >= 2 && !mbar_wait(smem_u32(&p_full[st]), ((g - 2) >> 1) & 1, d_err)) { ok = false; break; }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t kb = sK + (g % kTcStages) * kTcTile;
-#pragma unroll
-          for (int kk = 0; kk < kHD / 16; ++kk)
-            mma_bf16(tmem + kTcKeys * st, sdesc(sQ + kk * 32), sdesc(kb + kk * 32), idesc_s, kk > 0 ? 1u : 0u);
-          mma_commit(smem_u32(&s_full[st]));
-          if (j == r.n - 1) mma_commit(smem_u32(q_empty));
-          if (pv >= 0 && !issue_pv(pv, pv_first)) { ok = false; break; }
-          pv = g;
-          pv_first = j == 0;
-          // the item's last P V follows at once: the softmax's read of O
-          // does not wait for the next item's copies
-          if (j == r.n - 1) {
-            if (!issue_pv(pv, pv_first)) { ok = false; break; }
-            pv = -1;
-          }
-        }
-        if (ok && r.n == 0) mma_commit(smem_u32(q_empty));
-      }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-    }
-    if (lane == 0 && ok && pv >= 0) issue_pv(pv, pv_first);
-    __syncwarp();
-  } else {
-    // softmax: kTcSplit threads per query row, `part` of its keys and output each
-    static_assert(kTcPart % 32 == 0 && kTcPart <= 64 && (kTcOut == 16 || kTcOut == 32),
-                  "32-column TMEM loads of S, one load of O per thread");
-    const float sc = 1.4426950408889634f * rsqrtf((float)kHD);
-    const uint32_t lane_base = (uint32_t)(32 * quarter) << 16;
-    const int kb0 = kTcPart * part;               // first key of this thread's part of a tile
-    constexpr float kRescale = 8.f;
-    // this row's 16-byte chunks of P buffer 0 for keys kb0 .. kb0 + 31: atom
-    // kb0 / 64, chunks (kb0 % 64) / 8 + q at position chunk ^ (row % 8)
-    const uint32_t prow = sP + (kb0 >> 6) * (kTcP / 2) + row * 128;
-    const int chunk0 = (kb0 & 63) >> 3;
-    // this thread's output dims of the O accumulator in TMEM
-    const uint32_t o_addr = tmem + lane_base + 256 + kTcOut * part;
-    // A bounded wait that runs out marks the thread failed; the next
-    // OR-barrier tells its partner warp, and both leave the loops (the other
-    // pairs' waits then run out in turn).
-    bool failed = false;
-    auto wait_or_abort = [&](uint64_t* bar, uint32_t parity) {
-      if (!mbar_wait(smem_u32(bar), parity, d_err)) failed = true;
-    };
-    bool ok = true;
-    int g = 0, it = 0;
-    for (int w = item_at(0); ok && w >= 0; w = item_at(++it)) {
-      int q0, h, b;
-      item(w, &q0, &h, &b);
-      const TileRanges r = tile_ranges(a, q0, lane);
-      const RowVis v = row_vis(a, q0 + row);
-      // the visible keys kb0 + i (i < kTcPart) of a row as a bit mask: [lo, hi) relative to the tile
-      auto range_bits = [&](int lo, int hi) -> unsigned long long {
-        lo = max(lo - kb0, 0);
-        hi = min(hi - kb0, kTcPart);
-        if (hi <= lo) return 0ull;
-        const unsigned long long up = hi >= 64 ? ~0ull : ((1ull << hi) - 1ull);
-        return up & ~((1ull << lo) - 1ull);
-      };
-      // m: the row max the probabilities of the item's tiles so far are
-      // taken against (raised only when a tile's max exceeds it by more than
-      // 2^8, so P stays below 256); l: this thread's part of their sum
-      float m = -INFINITY, l = 0.f;
-      for (int j = 0; j < r.n; ++j, ++g) {
-        const int st = g & 1;
-        int kt, kend;
-        tile_at(r, j, &kt, &kend);
-        // visible keys of this part: the context prefix [0, ctx], the windows,
-        // none past the range's end (each key belongs to one range's tiles)
-        const int lim = min(kend - kt, kTcKeys);
-        const bool open = !a.dense && kt + kTcKeys - 1 < kend && kt + kTcKeys - 1 <= r.cmin && v.ctx >= 0;
-        unsigned long long vis = ~0ull;
-        if (!open)
-          vis = (range_bits(0, v.ctx - kt + 1) | range_bits(v.w1lo - kt, v.w1hi - kt) |
-                 range_bits(v.w2lo - kt, v.w2hi - kt)) &
-                range_bits(0, lim);
-        wait_or_abort(&s_full[st], (g >> 1) & 1);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        float sv[kTcPart];
-#pragma unroll
-        for (int c = 0; c < kTcPart / 32; ++c) tmem_ld32(tmem + lane_base + kTcKeys * st + kb0 + 32 * c, sv + 32 * c);
-        // raw scores: sc > 0, so the max commutes with the scaling
-        if (vis != ~0ull) {
-#pragma unroll
-          for (int e = 0; e < kTcPart; ++e) sv[e] = ((vis >> e) & 1ull) ? sv[e] : -INFINITY;
-        }
-        // four independent max chains, then combined
-        float mq[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-        for (int e = 0; e < kTcPart; e += 8)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) mq[c] = max3f(mq[c], sv[e + 2 * c], sv[e + 2 * c + 1]);
-        float mx = fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3]));
-        // the row's max over its parts (the partner warp)
-        s_mx[(st * kTcSplit + part) * kTcRows + row] = mx;
-        if (pair_bar_or(quarter, failed)) { ok = false; break; }
-        mx = s_mx[(st * kTcSplit) * kTcRows + row];
-#pragma unroll
-        for (int q = 1; q < kTcSplit; ++q) mx = fmaxf(mx, s_mx[(st * kTcSplit + q) * kTcRows + row]);
-        // A new reference max when this tile's exceeds it by more than 2^8: O
-        // and l so far are scaled to it (O once the previous tile's P V has
-        // landed; nothing is accumulated before a finite max).  The TMEM
-        // load and store are warp-wide: a warp rescales when any of its rows
-        // needs it, the others by 1.
-        const bool raise = mx * sc > m + kRescale;
-        const float f = (raise && m != -INFINITY) ? ex2(m - mx * sc) : 1.f;
-        if (__any_sync(0xffffffffu, f != 1.f)) {
-          wait_or_abort(&o_full[(g - 1) & 1], ((g - 1) >> 1) & 1);
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          float rr[kTcOut];
-          tmem_ld32(o_addr, rr);
-#pragma unroll
-          for (int d = 0; d < kTcOut; ++d) rr[d] *= f;
-          tmem_st32(o_addr, rr);
-        }
-        if (raise) {
-          l *= f;
-          m = mx * sc;
-        }
-        const float mn = m;
-        // P = exp2(S sc - mn) rounded to bf16 (ex2(-inf) = 0 for masked keys),
-        // the sum of the rounded values
-        const uint32_t pbase = prow + st * kTcP;
-        const float nmn = mn == -INFINITY ? 0.f : -mn;
-        const uint64_t sc2 = f2(sc, sc), nmn2 = f2(nmn, nmn);
-        uint64_t ps2[4] = {f2(0.f, 0.f), f2(0.f, 0.f), f2(0.f, 0.f), f2(0.f, 0.f)};   // independent sums
-#pragma unroll
-        for (int q = 0; q < kTcPart / 8; ++q) {
-          uint32_t pk[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int e = 8 * q + 2 * u;
-            const float2 arg = f2_split(fma_f2(f2(sv[e], sv[e + 1]), sc2, nmn2));
-            pk[u] = pack_bf16(ex2(arg.x), ex2(arg.y));
-            const float2 pf = unpack_bf16(pk[u]);
-            ps2[u] = add_f2(ps2[u], f2(pf.x, pf.y));
-          }
-          const uint32_t addr = pbase + (((chunk0 + q) ^ (row & 7)) << 4);
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]),
-                       "r"(pk[3])
-                       : "memory");
-        }
-        const float2 ps = f2_split(add_f2(add_f2(ps2[0], ps2[1]), add_f2(ps2[2], ps2[3])));
-        l += ps.x + ps.y;
-        // S_g read, P_g written: to the tensor cores (async proxy); every
-        // softmax thread arrives
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&p_full[st])) : "memory");
-      }
-      if (!ok) break;
-      float o[kTcOut];
-#pragma unroll
-      for (int d = 0; d < kTcOut; ++d) o[d] = 0.f;
-      if (r.n > 0) {
-        // the item's last P V completes the accumulator; once every softmax
-        // thread has read it, the next item's first P V may overwrite it
-        wait_or_abort(&o_full[(g - 1) & 1], ((g - 1) >> 1) & 1);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tmem_ld32(o_addr, o);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        if (pair_bar_or(quarter, failed)) { ok = false; break; }
-        asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(o_free)) : "memory");
-      }
-      // the row's sum over its parts, in a fixed order (one buffer per item
-      // parity: a thread writes the next item's sums only after the pair
-      // barrier below, which its partner passes after reading this item's)
-      float* sl = s_l + (it & 1) * kTcSplit * kTcRows;
-      sl[part * kTcRows + row] = l;
-      pair_bar(quarter);
-      float lt = 0.f;
-#pragma unroll
-      for (int q = 0; q < kTcSplit; ++q) lt += sl[q * kTcRows + row];
-      const int qi = q0 + row;
-      if (qi < a.q_end && lt > 0.f) {
-        const float inv = 1.f / lt;
-        float* dst =
-            a.out + (((size_t)b * (a.q_end - a.q_begin) + (qi - a.q_begin)) * a.H + h) * kHD + kTcOut * part;
-#pragma unroll
-        for (int d = 0; d < kTcOut; d += 4)
-          *reinterpret_cast<float4*>(dst + d) = make_float4(o[d] * inv, o[d + 1] * inv, o[d + 2] * inv, o[d + 3] * inv);
-      }
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-}
 
 }  // namespace kf
 
@@ -802,19 +417,45 @@ extern "C" int kf_op_train_attention(int32_t blocks, int32_t B, int32_t H, int32
   // head's 128 consecutive tokens (rows past T read as zero)
   const uint64_t dims[4] = {64, (uint64_t)H, (uint64_t)T, (uint64_t)B};
   const uint64_t strides[3] = {128, (uint64_t)H * 128, (uint64_t)T * H * 128};
-  const uint32_t box[4] = {64, 1, kTcRows, 1};
-  CUtensorMap mq, mk, mv;
-  if (!encode_map_bf16(&mq, q, 4, dims, strides, box) || !encode_map_bf16(&mk, kk, 4, dims, strides, box) ||
-      !encode_map_bf16(&mv, v, 4, dims, strides, box))
+  const uint32_t box[4] = {64, 1, fa::kRows, 1};
+  TrainPolicy::Maps maps;
+  if (!encode_map_bf16(&maps.q, q, 4, dims, strides, box) || !encode_map_bf16(&maps.k, kk, 4, dims, strides, box) ||
+      !encode_map_bf16(&maps.v, v, 4, dims, strides, box))
     return KF_E_CUDA;
+  // the query tiles that hold rows of [q_begin, q_end)
+  TrainArgs g{};
+  g.a = a;
+  g.n_batch = B;
+  g.qr = k <= fa::kRows ? fa::kRows / k * k : fa::kRows;
+  for (int p = 0; p <= blocks; ++p) {
+    const long long bs = p == 0 ? 0 : N + (long long)(p - 1) * N * k, len = p == 0 ? N : (long long)N * k;
+    const long long lo = std::max<long long>(q_begin, bs) - bs, hi = std::min<long long>(q_end, bs + len) - bs;
+    const int rows = p == 0 ? fa::kRows : g.qr;
+    if (hi <= lo) continue;
+    g.first[p] = (int)(lo / rows);
+    g.count[p] = (int)((hi + rows - 1) / rows) - g.first[p];
+    g.n_qt += g.count[p];
+  }
+  if (g.n_qt <= kTileList) {
+    // sorted by the context keys a tile's last row sees (the windows add about
+    // the same to every block tile)
+    std::vector<std::pair<long long, int>> tiles;
+    for (int p = 0; p <= blocks; ++p)
+      for (int i = g.first[p]; i < g.first[p] + g.count[p]; ++i) {
+        const long long bs = p == 0 ? 0 : N + (long long)(p - 1) * N * k, q0 = bs + (long long)i * (p == 0 ? fa::kRows : g.qr);
+        tiles.push_back({p == 0 ? q0 + fa::kRows : (q0 - bs + g.qr) / k + (long long)fa::kKeys * p, (int)q0});
+      }
+    std::stable_sort(tiles.begin(), tiles.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+    for (int i = 0; i < g.n_qt; ++i) g.q0[i] = tiles[i].second;
+  }
+  const long long items = (long long)g.n_qt * H * B;
+  if (items > (1ll << 30)) return KF_E_ARG;
   int* err = op_error_word(s);
   if (!err) return KF_E_CUDA;
   static PerDevice attr_tc;
-  set_smem_attr(attr_tc, k_train_attention_tc, tc_smem_bytes());
-  // persistent: one CTA per SM over the (query tile, head, sequence) items
-  const long long items = (long long)ceil_div(q_end - q_begin, kTcRows) * H * B;
-  if (items > (1ll << 30)) return KF_E_ARG;
-  const dim3 grid((unsigned)std::min<long long>(items, device_sms()));
-  kf_launch(k_train_attention_tc, grid, dim3(kTcThreads), tc_smem_bytes(), s, mq, mk, mv, a, (int)B, err);
+  set_smem_attr(attr_tc, fa::k_attn_tc<TrainPolicy>, fa::kSmemBytes);
+  // persistent: two CTAs per SM over the (query tile, head, sequence) items
+  const dim3 grid((unsigned)std::min<long long>(items, 2ll * device_sms()));
+  kf_launch(fa::k_attn_tc<TrainPolicy>, grid, dim3(fa::kThreads), fa::kSmemBytes, s, maps, g, err);
   return cudaGetLastError() == cudaSuccess ? KF_OK : KF_E_CUDA;
 }
