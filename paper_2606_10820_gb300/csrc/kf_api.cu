@@ -259,15 +259,19 @@ static void attn_plan_mma(kf_ctx* c, int n_groups, int R, int* n_split, int* kps
 // the producers of x, and the QKV and MLP-up epilogues scale their rows (the
 // gains are folded into wqkv and w_up).  Otherwise an RMSNorm kernel writes
 // the normed rows into xn.
-static void enqueue_layers(kf_ctx* c, int R, int n_groups, const int4* groups, int uniform_rows) {
+// groups (prefill): group_rows-row groups of consecutive rows; NULL (decode):
+// uniform_rows rows per sequence.
+static void enqueue_layers(kf_ctx* c, int R, int n_groups, const int4* groups, int group_rows, int uniform_rows) {
   const int d = c->d, H = c->H, F = c->F;
   cudaStream_t s = c->stream;
   // Attention: the warp-MMA kernel for the bf16 cache with head_dim 64; the
   // FP32-FMA kernel otherwise (fp32 cache, head_dim 32).
-  const int rows = groups ? kMaxGroupRows : uniform_rows;
-  const bool mma_attn = attention_mma_supported(c->bf16, c->hd, rows);
-  int n_split, kps;
-  if (mma_attn) attn_plan_mma(c, n_groups, R, &n_split, &kps);
+  const int rows = groups ? group_rows : uniform_rows;
+  const bool tile_attn = groups && group_rows > kMaxGroupRows;
+  const bool mma_attn = !tile_attn && attention_mma_supported(c->bf16, c->hd, rows);
+  int n_split = 1, kps = 0;
+  if (tile_attn) {}
+  else if (mma_attn) attn_plan_mma(c, n_groups, R, &n_split, &kps);
   else attn_plan(c, n_groups, R, 1 << 30, &n_split, &kps);
   auto norm_in = [&](Epi& e) {
     e.ss_in = c->ss; e.nslot = d / 64; e.inv_d = 1.0f / d; e.eps = c->cfg.rms_eps;
@@ -326,10 +330,13 @@ static void enqueue_layers(kf_ctx* c, int R, int n_groups, const int4* groups, i
     a.split_count = c->split_count;
     prof_begin(c, KF_KIND_ATTENTION);
     bool merged = false;
-    if (mma_attn) {
+    if (tile_attn) {
+      if (launch_attention_prefill(a, n_groups, s) != 0) c->launch_failed = true;
+    } else if (mma_attn) {
       if (launch_attention_mma(a, n_groups, rows, c->cfg.max_len, s, &merged) != 0) c->launch_failed = true;
+    } else {
+      launch_attention(c->bf16, a, n_groups, c->cfg.max_len, s);
     }
-    else launch_attention(c->bf16, a, n_groups, c->cfg.max_len, s);
     prof_end(c);
     if (n_split > 1 && !merged) {
       prof_begin(c, KF_KIND_ATTN_COMBINE);
@@ -406,7 +413,7 @@ static void enqueue_step(kf_ctx* c, int B, int P, int k, const float* noise) {
     gemm(c, KF_KIND_NOISE_GEMM, B * kz, d, c->NH, c->nhid, c->NH, c->ne_w2, c->NH, e2,
          pf ? c->layers[0].wqkv : nullptr, (size_t)3 * d * d * c->esz);
   }
-  enqueue_layers(c, R, B, nullptr, S);
+  enqueue_layers(c, R, B, nullptr, 0, S);
   prof_begin(c, KF_KIND_HEAD_NORM);
   launch_rmsnorm(c->bf16, nh, c->head_map, c->x, d, c->final_norm, c->cfg.rms_eps, c->head_in, s);
   prof_end(c);
@@ -697,8 +704,25 @@ int kf_init(const kf_config* cfg_in, const kf_weights* w, void* stream, kf_ctx**
 }
 
 // Prefill: the KV of each listed slot's first n tokens (positions 0..n-1),
-// in row chunks of up to prefill_rows, attention groups of <= 16 rows per
-// sequence.  The slots' pages must be allocated and uploaded.
+// in row chunks of up to prefill_rows, attention groups of consecutive rows of a
+// sequence: up to 128 for the tcgen05 kernel, else up to 16.  The slots' pages
+// must be allocated and uploaded.
+// The rows of a chunk's attention groups: 128 (tcgen05) once the 128-row items
+// cover the SMs and hold 40 rows or more on average, else 16 (warp-level MMA, which
+// also splits the keys of few long rows).  Measured, 768-wide model, 4 layers,
+// 16-row -> 128-row groups, microseconds per prefill: 16 prompts of 128-896
+// 1334 -> 1196, 64 of 64 530 -> 487, 64 of 48 441 -> 424, 4 of 400 (192 items) 355
+// -> 344; but 64 of 32 364 -> 368, 64 of 17 284 -> 300, 16 of 32 221 -> 235, one of
+// 1000 (96 items) 312 -> 344, 4 of 128 (48 items) 218 -> 239.
+static int prefill_group_rows(const kf_ctx* c, const std::vector<int4>& runs) {
+  if (!c->bf16 || c->hd != 64) return kMaxGroupRows;
+  long long rows = 0, tiles = 0;
+  for (const int4& u : runs) {
+    rows += u.z;
+    tiles += ceil_div(u.z, kMaxTileRows);
+  }
+  return tiles * c->H >= c->num_sms && rows >= 40 * tiles ? kMaxTileRows : kMaxGroupRows;
+}
 struct PrefillSeq {
   int slot;
   const int32_t* tok;
@@ -706,10 +730,16 @@ struct PrefillSeq {
 };
 static int prefill_rows(kf_ctx* c, const std::vector<PrefillSeq>& seqs) {
   std::vector<int32_t> r_tok, r_seq, r_pos;
-  std::vector<int4> grp;
+  std::vector<int4> runs, grp;     // runs: {slot, first row, rows, first position} in the chunk
   auto flush = [&]() -> int {
     int R = (int)r_tok.size();
     if (R == 0) return KF_OK;
+    const int group_rows = prefill_group_rows(c, runs);
+    for (const int4& u : runs)
+      for (int i = 0; i < u.z; i += group_rows)
+        grp.push_back(make_int4(u.x, u.y + i, std::min(group_rows, u.z - i), u.w + i));
+    if (group_rows > kMaxGroupRows)     // most keys first
+      std::stable_sort(grp.begin(), grp.end(), [](const int4& x, const int4& y) { return x.w + x.z > y.w + y.z; });
     KF_CUDA(cudaMemcpyAsync(c->row_tok, r_tok.data(), R * 4, cudaMemcpyHostToDevice, c->stream));
     KF_CUDA(cudaMemcpyAsync(c->row_seq, r_seq.data(), R * 4, cudaMemcpyHostToDevice, c->stream));
     KF_CUDA(cudaMemcpyAsync(c->row_pos, r_pos.data(), R * 4, cudaMemcpyHostToDevice, c->stream));
@@ -721,20 +751,20 @@ static int prefill_rows(kf_ctx* c, const std::vector<PrefillSeq>& seqs) {
       launch_embed_tokens(c->bf16, R, c->row_tok, c->tok_emb, c->pos_emb, c->row_pos, c->V, c->d,
                           c->x, c->fused ? c->xn : nullptr, c->fused ? c->ss : nullptr, c->d_err,
                           c->stream);
-      enqueue_layers(c, R, (int)grp.size(), c->groups, 0);
+      enqueue_layers(c, R, (int)grp.size(), c->groups, group_rows, 0);
     }
     KF_CUDA(enqueue_status(c));
     // the host vectors are reused: wait until the copies have consumed them
     KF_CUDA(cudaStreamSynchronize(c->stream));
-    r_tok.clear(); r_seq.clear(); r_pos.clear(); grp.clear();
+    r_tok.clear(); r_seq.clear(); r_pos.clear(); runs.clear(); grp.clear();
     return KF_OK;
   };
   for (const PrefillSeq& q : seqs) {
     int p = 0;
     while (p < q.n) {
       if ((int)r_tok.size() == c->prefill_rows) KF_TRY(flush());
-      int take = std::min({q.n - p, kMaxGroupRows, c->prefill_rows - (int)r_tok.size()});
-      grp.push_back(make_int4(q.slot, (int)r_tok.size(), take, 0));
+      int take = std::min(q.n - p, c->prefill_rows - (int)r_tok.size());
+      runs.push_back(make_int4(q.slot, (int)r_tok.size(), take, p));
       for (int i = 0; i < take; ++i) {
         r_tok.push_back(q.tok[p + i]);
         r_seq.push_back(q.slot);

@@ -495,6 +495,12 @@ bool attention_mma_supported(bool bf16, int hd, int rows);
 int launch_attention_mma(const AttnArgs& a, int n_groups, int rows, int max_keys, cudaStream_t s,
                          bool* merged);
 
+// prefill attention on tcgen05 (bf16 cache, head_dim 64): a.groups holds
+// {slot, first row, rows <= 128, first position} of consecutive rows, most keys
+// first; -1 if the TMA map is refused
+constexpr int kMaxTileRows = 128;
+int launch_attention_prefill(const AttnArgs& a, int n_groups, cudaStream_t s);
+
 // the op entry points' error word on the current device, cleared on s
 // (read back by kf_op_status); nullptr on failure
 int* op_error_word(cudaStream_t s);
