@@ -183,13 +183,6 @@ static int dalloc(kf_ctx* c, T** p, size_t bytes, bool zero = true) {
   } while (0)
 
 // ------------------------------------------------------------- launches
-// programmatic dependent launch for the kernels enqueued in this scope
-struct PdlScope {
-  bool prev;
-  explicit PdlScope(bool on) : prev(g_pdl) { g_pdl = on; }
-  ~PdlScope() { g_pdl = prev; }
-};
-
 static void prof_begin(kf_ctx* c, int kind) {
   if (!c->prof) return;
   if (c->ev_used + 2 > (int)c->ev.size()) return;

@@ -104,7 +104,7 @@ int launch_attention_prefill(const AttnArgs& a, int n_groups, cudaStream_t s) {
   const long long items = (long long)n_groups * a.H;
   if (items > (1ll << 30)) return -1;
   const dim3 grid((unsigned)std::min<long long>(items, 2ll * device_sms()));
-  kf_launch(fa::k_attn_tc<PrefillPolicy>, grid, dim3(fa::kThreads), fa::kSmemBytes, s, maps, p, a.d_err);
+  kf_launch(fa::k_attn_tc<PrefillPolicy>, grid, dim3(fa::kThreads), fa::kSmemBytes, s, maps, p, a.d_err, 0);
   return 0;
 }
 

@@ -113,7 +113,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //   store(a, it, row, o, inv)   the finished row
 template <class P>
 __global__ void __launch_bounds__(kThreads, 2)
-k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args a, int* d_err) {
+k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args a, int* d_err, int clear_err) {
   extern __shared__ __align__(1024) uint8_t sm[];
   const uint32_t sQ = smem_u32(sm);
   const uint32_t sK = sQ + kTileBytes;
@@ -132,6 +132,8 @@ k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args 
   uint64_t* o_free = s_full + 4;                // the item's O is in registers
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 5);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  // (the word is set below, or after a wait of about 2 s)
+  if (clear_err && t == 0 && blockIdx.x == 0) atomicExch(d_err, 0);
   if (sQ & 1023) {                              // (uniform) swizzle atoms need the alignment
     if (t == 0) atomicOr(d_err, kErrInternal);
     return;

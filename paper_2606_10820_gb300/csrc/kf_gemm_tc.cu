@@ -60,8 +60,13 @@ struct TcArgs {
   const char* l2_next;   // the next projection's weights, prefetched into L2 (or NULL)
   unsigned long long l2_bytes;
   int* d_err;
+  int clear_err;      // the first CTA zeroes *d_err
   Epi epi;
 };
+
+__device__ __forceinline__ void clear_error(const TcArgs& g) {
+  if (g.clear_err && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) atomicExch(g.d_err, 0);
+}
 
 __device__ __forceinline__ void epi_bar() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
@@ -334,6 +339,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
   const int nkb = kb1 - kb0;                  // K atoms of this split
   const int nst = (nkb + AT - 1) / AT;        // pipeline stages (the last may be short)
 
+  clear_error(g);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(smem_u32(&bars[s]), 1);
@@ -641,6 +647,7 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   auto tile_m0 = [&](int t) { return (EPI == EPI_HEAD ? t % m_tiles : t / n_tiles) * kBM; };
   auto tile_n0 = [&](int t) { return (EPI == EPI_HEAD ? t / m_tiles : t % n_tiles) * BN; };
   const int nkb = g.K / kBK;
+  clear_error(g);
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
@@ -831,6 +838,7 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   auto tile_m0 = [&](int t) { return (EPI == EPI_HEAD ? t % m_tiles : t / n_tiles) * 2 * kBM + (int)rank * kBM; };
   auto tile_n0 = [&](int t) { return (EPI == EPI_HEAD ? t / m_tiles : t % n_tiles) * BN; };
   const int nkb = g.K / kBK;
+  clear_error(g);
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
@@ -1089,7 +1097,7 @@ static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s
   const bool pf = g.l2_next && g.l2_bytes >= 16 && !(reinterpret_cast<uintptr_t>(g.l2_next) & 15);
   a.l2_next = pf ? static_cast<const char*>(g.l2_next) : nullptr;
   a.l2_bytes = pf ? (g.l2_bytes & ~(size_t)15) : 0;
-  a.d_err = d_err; a.epi = g.epi;
+  a.d_err = d_err; a.clear_err = g.clear_err; a.epi = g.epi;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_tiles, m_tiles, splits);
   cfg.blockDim = dim3(kThreads);
@@ -1128,7 +1136,7 @@ static int launch_persist_epi(const GemmDesc& g, int* d_err, int num_sms, cudaSt
   a.M = g.M; a.N = g.N; a.K = g.K; a.kb_per_split = g.K / kBK; a.splits = 1;
   a.a_box = (uint32_t)a_rows * kBK * 2;
   a.l2_next = nullptr; a.l2_bytes = 0;
-  a.d_err = d_err; a.epi = g.epi;
+  a.d_err = d_err; a.clear_err = g.clear_err; a.epi = g.epi;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(tiles, num_sms));
   cfg.blockDim = dim3(kPersistWarps * 32);
@@ -1170,7 +1178,7 @@ static int launch_pair_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStrea
   a.M = g.M; a.N = g.N; a.K = g.K; a.kb_per_split = g.K / kBK; a.splits = 1;
   a.a_box = 0;
   a.l2_next = nullptr; a.l2_bytes = 0;
-  a.d_err = d_err; a.epi = g.epi;
+  a.d_err = d_err; a.clear_err = g.clear_err; a.epi = g.epi;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * std::min(tiles, num_sms / 2));
   cfg.blockDim = dim3(kPairThreads);

@@ -404,6 +404,12 @@ __device__ __forceinline__ void pdl_wait() {
 }
 
 extern thread_local bool g_pdl;   // launch with the programmatic-serialization attribute
+// programmatic dependent launch for the kernels enqueued in this scope
+struct PdlScope {
+  bool prev;
+  explicit PdlScope(bool on) : prev(g_pdl) { g_pdl = on; }
+  ~PdlScope() { g_pdl = prev; }
+};
 // tensor-core GEMM launch options for the launches made by this thread
 constexpr int kGemmNoPersist = 1;  // one CTA per tile even past a wave of tiles
 extern thread_local int g_gemm_flags;
@@ -435,6 +441,10 @@ struct GemmDesc {
   // prefetch them into L2 at their start (16-byte aligned), or NULL
   const void* l2_next = nullptr;
   size_t l2_bytes = 0;
+  // the tensor-core kernel clears the error word as it starts (the op entry
+  // points: a clearing memset of its own before each call cost about 2 us).
+  // Its kernels set the word only after a wait of about 2 s
+  bool clear_err = false;
 };
 
 // SIMT GEMM (bf16 operands; fp32 accumulation, k ascending per output)
@@ -501,9 +511,9 @@ int launch_attention_mma(const AttnArgs& a, int n_groups, int rows, int max_keys
 constexpr int kMaxTileRows = 128;
 int launch_attention_prefill(const AttnArgs& a, int n_groups, cudaStream_t s);
 
-// the op entry points' error word on the current device, cleared on s
-// (read back by kf_op_status); nullptr on failure
-int* op_error_word(cudaStream_t s);
+// the op entry points' error word on the current device, cleared on s unless
+// the call's kernel does it (read back by kf_op_status); nullptr on failure
+int* op_error_word(cudaStream_t s, bool clear = true);
 
 // message for kf_last_error(NULL) (calls without a context)
 void set_global_error(const std::string& msg);

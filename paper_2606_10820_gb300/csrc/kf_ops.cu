@@ -43,9 +43,9 @@ int ensure_err(int dev) {
 }  // namespace
 
 namespace kf {
-// the calling thread's device's op error word, cleared on `s` (kf_op_status
-// reads it); nullptr if it cannot be had
-int* op_error_word(cudaStream_t s) {
+// the calling thread's device's op error word, with `clear` cleared on `s`
+// (kf_op_status reads it); nullptr if it cannot be had
+int* op_error_word(cudaStream_t s, bool clear) {
   int dev = 0;
   if (current_device(&dev) != KF_OK) return nullptr;
   int* err = nullptr;
@@ -54,7 +54,7 @@ int* op_error_word(cudaStream_t s) {
     if (ensure_err(dev) != KF_OK) return nullptr;
     err = g_ops[dev].err;
   }
-  if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return nullptr;
+  if (clear && cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return nullptr;
   return err;
 }
 }  // namespace kf
@@ -71,8 +71,11 @@ static int head_tokens(int32_t rows, int32_t V, int32_t d, const void* x, const 
   g.epi.rec = rec;
   g.epi.nchunk = nchunk;
   g.epi.want_arg = map_kind == KF_MAP_ARGMAX;
+  g.clear_err = true;
   if (!tc_gemm_supported(g)) return KF_E_ARG;
   if (launch_gemm_tc(g, err, s) != 0) return KF_E_CUDA;
+  // the token selection waits for the records itself: its launch overlaps them
+  const PdlScope pdl(true);
   launch_head_select(true, rows, rec, nchunk, x, d, w_head, V, 1.0f / tau, map_kind, noise, tokens, 0, 0,
                      err, StepCommit{}, s);
   return cudaGetLastError() == cudaSuccess ? KF_OK : KF_E_CUDA;
@@ -95,16 +98,9 @@ extern "C" int kf_op_gemm_bf16(int32_t impl, int32_t M, int32_t N, int32_t K, co
   if (impl == KF_GEMM_TCGEN05 || impl == KF_GEMM_TCGEN05_PER_TILE) {
     if (!tc_gemm_supported(g)) return KF_E_ARG;
     g_gemm_flags = impl == KF_GEMM_TCGEN05_PER_TILE ? kGemmNoPersist : 0;
-    int dev = 0;
-    if (current_device(&dev) != KF_OK) return KF_E_CUDA;
-    int* err = nullptr;
-    {
-      std::lock_guard<std::mutex> lock(g_ops_mu);
-      if (ensure_err(dev) != KF_OK) return KF_E_CUDA;
-      err = g_ops[dev].err;
-    }
-    // each call starts with a clear error word (kf_op_status reads it)
-    if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) return KF_E_CUDA;
+    int* err = op_error_word(s, false);
+    if (!err) return KF_E_CUDA;
+    g.clear_err = true;
     if (launch_gemm_tc(g, err, s) != 0) return KF_E_CUDA;
   } else if (impl == KF_GEMM_SKINNY) {
     if (!skinny_gemm_supported(g)) return KF_E_ARG;
@@ -148,7 +144,6 @@ extern "C" int kf_op_head_tokens(int32_t rows, int32_t V, int32_t d, const void*
     }
     sc.rec_bytes = need;
   }
-  if (cudaMemsetAsync(sc.err, 0, sizeof(int), s) != cudaSuccess) return KF_E_CUDA;
   return head_tokens(rows, V, d, x, w_head, noise, tau, map_kind, tokens, sc.rec, sc.err, s);
 }
 
@@ -201,9 +196,8 @@ extern "C" int kf_op_head_tokens_noalloc(int32_t rows, int32_t V, int32_t d, con
     sc = g_noalloc[dev];
   }
   cudaStream_t s = (cudaStream_t)stream;
-  // the error word keeps the previous call's value: clear it (the records
-  // need no clearing, every one this call reads it writes first)
-  if (cudaMemsetAsync(sc.err, 0, sizeof(int), s) != cudaSuccess) return KF_E_CUDA;
+  // the error word keeps the previous call's value: the GEMM clears it (the
+  // records need no clearing, every one this call reads it writes first)
   return head_tokens(rows, V, d, x, w_head, noise, tau, map_kind, tokens, sc.rec, sc.err, s);
 }
 
