@@ -1043,18 +1043,23 @@ bool tc_gemm_supported(const GemmDesc& g) {
   return get_encode();
 }
 
+// K splits over a cluster of up to 8 CTAs when the tiles alone leave SMs idle:
+// the largest power of two that keeps one CTA per SM and two K blocks per split
+// (odd cluster sizes measured slower; QKV only within one M tile: at 256 rows
+// its 2-way split measured slower)
+static int k_splits(int epi, int tiles, int m_tiles, int kb_total, int num_sms, int most) {
+  int splits = 1;
+  if (epi != EPI_HEAD && (epi != EPI_QKV || m_tiles == 1))
+    while (splits < most && tiles * splits * 2 <= num_sms && kb_total >= splits * 4) splits *= 2;
+  return splits;
+}
+
 template <int BN, int STAGES, int EPI, int AT>
-static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s) {
+static int launch_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s, int most_splits = 8) {
   const int n_tiles = ceil_div(g.N, BN), m_tiles = ceil_div(g.M, kBM);
   const int tiles = n_tiles * m_tiles;
   const int kb_total = g.K / kBK;
-  // split K over a cluster of up to 8 CTAs when the tiles alone leave SMs
-  // idle: the largest power of two that keeps one wave and two K blocks per
-  // split (odd cluster sizes measured slower)
-  // (QKV only within one M tile: at 256 rows its 2-way split measured slower)
-  int splits = 1;
-  if (EPI != EPI_HEAD && (EPI != EPI_QKV || m_tiles == 1))
-    while (splits < 8 && tiles * splits * 2 <= num_sms && kb_total >= splits * 4) splits *= 2;
+  int splits = k_splits(EPI, tiles, m_tiles, kb_total, num_sms, most_splits);
   int kbps = ceil_div(kb_total, splits);
   splits = ceil_div(kb_total, kbps);   // no empty splits
   const size_t smem = (size_t)STAGES * AT * (kBM * kBK * 2 + BN * kBK * 2) + 1024 + 256 + sizeof(EpiMeta);
@@ -1193,17 +1198,45 @@ static int launch_pair_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStrea
 }
 
 template <int BN, int STAGES, int AT>
-static int launch_bn(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s) {
+static int launch_bn(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s, int most_splits = 8) {
   switch (g.epi.kind) {
-    case EPI_STORE: return launch_epi<BN, STAGES, EPI_STORE, AT>(g, d_err, num_sms, s);
-    case EPI_BIAS_GELU: return launch_epi<BN, STAGES, EPI_BIAS_GELU, AT>(g, d_err, num_sms, s);
-    case EPI_RESID: return launch_epi<BN, STAGES, EPI_RESID, AT>(g, d_err, num_sms, s);
-    case EPI_NOISE_OUT: return launch_epi<BN, STAGES, EPI_NOISE_OUT, AT>(g, d_err, num_sms, s);
-    case EPI_LOGITS: return launch_epi<BN, STAGES, EPI_LOGITS, AT>(g, d_err, num_sms, s);
-    case EPI_STORE_F32: return launch_epi<BN, STAGES, EPI_STORE_F32, AT>(g, d_err, num_sms, s);
-    case EPI_QKV: return launch_epi<BN, STAGES, EPI_QKV, AT>(g, d_err, num_sms, s);
+    case EPI_STORE: return launch_epi<BN, STAGES, EPI_STORE, AT>(g, d_err, num_sms, s, most_splits);
+    case EPI_BIAS_GELU: return launch_epi<BN, STAGES, EPI_BIAS_GELU, AT>(g, d_err, num_sms, s, most_splits);
+    case EPI_RESID: return launch_epi<BN, STAGES, EPI_RESID, AT>(g, d_err, num_sms, s, most_splits);
+    case EPI_NOISE_OUT: return launch_epi<BN, STAGES, EPI_NOISE_OUT, AT>(g, d_err, num_sms, s, most_splits);
+    case EPI_LOGITS: return launch_epi<BN, STAGES, EPI_LOGITS, AT>(g, d_err, num_sms, s, most_splits);
+    case EPI_STORE_F32: return launch_epi<BN, STAGES, EPI_STORE_F32, AT>(g, d_err, num_sms, s, most_splits);
+    case EPI_QKV: return launch_epi<BN, STAGES, EPI_QKV, AT>(g, d_err, num_sms, s, most_splits);
   }
   return -1;
+}
+
+// clusters of cs CTAs that run at the same time on the current device, at one
+// CTA per SM (every k_gemm_tc takes more than half of an SM's shared memory): a
+// cluster lies within a GPC, so fewer than num_sms / cs (152 SMs: 76, 36 and 15
+// clusters of 2, 4 and 8)
+static int active_clusters(int cs) {
+  static PerDevice pd[9];
+  return (int)per_device(pd[cs], [&] {
+    constexpr size_t smem = (size_t)4 * 2 * (kBM * kBK * 2 + 64 * kBK * 2) + 1024 + 256 + sizeof(EpiMeta);
+    static PerDevice attr;
+    set_smem_attr(attr, k_gemm_tc<64, 4, EPI_STORE_F32, 2>, smem);
+    cudaLaunchConfig_t q = {};
+    q.gridDim = dim3(1, 1, cs);
+    q.blockDim = dim3(kThreads);
+    q.dynamicSmemBytes = smem;
+    cudaLaunchAttribute ca;
+    ca.id = cudaLaunchAttributeClusterDimension;
+    ca.val.clusterDim.x = 1; ca.val.clusterDim.y = 1; ca.val.clusterDim.z = cs;
+    q.attrs = &ca;
+    q.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_gemm_tc<64, 4, EPI_STORE_F32, 2>, &q) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    return (long long)n;
+  });
 }
 
 int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
@@ -1255,7 +1288,19 @@ int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
                           ceil_div(g.N, 64) * m_tiles * 4 > num_sms &&      // 64-wide: split 2 at most
                           ceil_div(g.N, 128) * m_tiles * 4 <= num_sms;      // 128-wide: split 4
   if (deep_split) return launch_bn<128, 3, 2>(g, d_err, num_sms, s);
-  if (ceil_div(g.N, 64) * m_tiles <= num_sms) return launch_bn<64, 4, 2>(g, d_err, num_sms, s);
+  if (ceil_div(g.N, 64) * m_tiles <= num_sms) {
+    // 64-wide tiles whose clusters do not all run at once, where 128-wide ones
+    // with the same K split do: the second wave costs more than the narrower
+    // spread gives (77 x 2308 x 832, 37 clusters of 4 where 36 fit, 9.3 -> 6.1
+    // us; 40 x 1024 x 1024, 16 of 8 where 15 fit, 8.3 -> 5.4; 40 x 1024 x 4096
+    // 12.0 -> 7.0).  The same split keeps the sums' lengths.
+    const int t64 = ceil_div(g.N, 64) * m_tiles, t128 = ceil_div(g.N, 128) * m_tiles, kb = g.K / kBK;
+    const int sp = k_splits(g.epi.kind, t64, m_tiles, kb, num_sms, 8);
+    if (sp > 1 && t64 > active_clusters(sp) && t128 <= active_clusters(sp) &&
+        k_splits(g.epi.kind, t128, m_tiles, kb, num_sms, sp) == sp)
+      return launch_bn<128, 3, 2>(g, d_err, num_sms, s, sp);
+    return launch_bn<64, 4, 2>(g, d_err, num_sms, s);
+  }
   if (ceil_div(g.N, 128) * m_tiles <= num_sms) return launch_bn<128, 3, 2>(g, d_err, num_sms, s);
   // More than a wave of 256-wide tiles: a persistent loop whose epilogues
   // overlap the next tile's mainloop (OWT-shaped batch 512, k = 4: QKV 35.1 ->
