@@ -799,16 +799,44 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
 // Why pairs: shared memory (128 B per clock) bounds the mainloop.  Per 64 of K
 // (512 clocks of MMA at 128 rows x 256 columns per SM) the one-CTA tile writes
 // and reads 48 KB each, 192 B per clock, and measures 0.40 us; a pair's CTA
-// writes and reads 32 KB each, and measures 0.28 us, the tensor cores' rate.
-// Measured, one-CTA loop -> pairs: LM-head records 2048 x 50,257 x 768 119 ->
-// 105 us (with the earlier record epilogue 147); fp32 products 8192 x 4096 x
-// 4096 191 -> 168 us (1.63 PFLOP/s), 4096 x 4096 x 1024 39.0 -> 37.0.
-// With K = 768 and two rounds of tiles the fill (2.4 us) and the last
-// epilogue (4 us) weigh as much as the mainloops, and the projections of a
-// step gain nothing (QKV 26.8 -> 28.4 us at 4096 rows): they stay on the
-// one-CTA kernels.  So do narrower pair tiles (256 x 192 and 256 x 128: slower
-// at every size tried).
+// writes and reads 32 KB each, and measures 0.28 us, the tensor cores' rate
+// (figures per shape at the dispatch rule).  With K = 768 and two rounds of tiles
+// the fill (2.4 us) and the last epilogue weigh as much as the mainloops, and
+// QKV (26.3 against 26.4 us at 4096 rows), the O projection and MLP-down (one
+// round; 17.3 against 19.5 us, 26.7 against 29.6) gain nothing: they stay on the
+// one-CTA kernels.  So do narrower pair tiles (256 x 192 and 256 x 128: slower at
+// every size tried).
 constexpr int kPairThreads = 64 + 32 * kEpiWarps;
+
+// Epilogues in which a thread keeps the row of its TMEM lane and stores whole
+// 32-byte sectors of it straight from its registers: the transposing epilogue's
+// writes and reads of its staging blocks take shared-memory bandwidth from the
+// next tile's mainloop (6.0 against 4.1 us per tile at K = 768).
+__host__ __device__ constexpr bool pair_row_epi(int epi) { return epi == EPI_STORE_F32 || epi == EPI_BIAS_GELU; }
+// 32 bytes (one sector) of global memory
+__device__ __forceinline__ void st_v8(void* p, const uint32_t* r) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+__device__ __forceinline__ uint32_t pack2(float x, float y) {
+  const __nv_bfloat162 t = __floats2bfloat162_rn(x, y);
+  return *reinterpret_cast<const uint32_t*>(&t);
+}
+// 32 consecutive floats of a row; as bf16
+__device__ __forceinline__ void st_row_f32(float* p, const float* v) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) st_v8(p + 8 * q, reinterpret_cast<const uint32_t*>(v) + 8 * q);
+}
+__device__ __forceinline__ void st_row_bf16(__nv_bfloat16* p, const float* v) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    uint32_t u[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) u[j] = pack2(v[16 * q + 2 * j], v[16 * q + 2 * j + 1]);
+    st_v8(p + 16 * q, u);
+  }
+}
 
 template <int BN, int STAGES, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
@@ -816,10 +844,10 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   constexpr uint32_t A_ATOM = kBM * kBK * 2;
   constexpr uint32_t B_ATOM = BN / 2 * kBK * 2;
   constexpr uint32_t STAGE_BYTES = A_ATOM + B_ATOM;
-  constexpr uint32_t STG_BYTES = EPI == EPI_HEAD ? 0 : kEpiWarps * 32 * 68 * 4;
+  constexpr uint32_t STG_BYTES = EPI == EPI_LOGITS ? kEpiWarps * 32 * 68 * 4 : 0;
   constexpr int TMEM_COLS = tmem_alloc_cols(2 * BN);
-  static_assert(EPI == EPI_HEAD || EPI == EPI_LOGITS || EPI == EPI_STORE_F32, "epilogues without per-row data");
-  static_assert(BN % 128 == 0 && BN <= 256 && STAGE_BYTES % 1024 == 0, "half the W rows per CTA, swizzle atoms aligned");
+  static_assert(pair_row_epi(EPI) || EPI == EPI_HEAD || EPI == EPI_LOGITS, "row epilogues, records, logits");
+  static_assert(BN % 64 == 0 && BN >= 128 && BN <= 256 && STAGE_BYTES % 1024 == 0, "half the W rows per CTA, swizzle atoms aligned");
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -938,13 +966,46 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     for (int t = pair; t < tiles; t += pairs, ++ti) {
       const uint32_t buf = ti & 1;
       const int m0 = tile_m0(t), n0 = tile_n0(t);
+      const int row = m0 + quarter * 32 + lane;
+      const bool in = row < g.M;
+      float rinv = 1.f;                           // while the mainloop runs
+      if (EPI == EPI_BIAS_GELU && g.epi.ss_in) rinv = in ? row_rinv(g.epi, row) : 0.f;
       const bool ok = mbar_wait_cluster(smem_u32(&accf[buf]), (ti >> 1) & 1, g.d_err);
       if (!__all_sync(0xffffffffu, ok)) break;    // timed out: the leader stops too
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t acc = tmem + buf * BN + ((uint32_t)(quarter * 32) << 16);
       if (EPI == EPI_HEAD) {
-        head_row(g, acc, m0 + quarter * 32 + lane, n0, ch * (BN / 2), (ch + 1) * (BN / 2));
-      } else if (m0 + quarter * 32 < g.M) {
+        head_row(g, acc, row, n0, ch * (BN / 2), (ch + 1) * (BN / 2));
+      } else if (m0 + quarter * 32 >= g.M) {      // (warp-uniform)
+      } else if (pair_row_epi(EPI)) {
+#pragma unroll 1
+        for (int c = ch * 64; c < BN && n0 + c < g.N; c += 128) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int col = n0 + c + 32 * h;
+            float v[32];
+            tmem_ld32(acc + c + 32 * h, v);
+            if (EPI == EPI_BIAS_GELU) {
+              if (g.epi.ss_in) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) v[j] *= rinv;
+              }
+              if (g.epi.bias) {
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                  const float4 bi = __ldg(reinterpret_cast<const float4*>(g.epi.bias + col + j));
+                  v[j] += bi.x; v[j + 1] += bi.y; v[j + 2] += bi.z; v[j + 3] += bi.w;
+                }
+              }
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = gelu_tanh_bf16(v[j]);
+              if (in) st_row_bf16(reinterpret_cast<__nv_bfloat16*>(g.epi.out) + (size_t)row * g.epi.ldo + col, v);
+            } else if (in) {
+              st_row_f32(g.epi.outf + (size_t)row * g.epi.ldo + col, v);
+            }
+          }
+        }
+      } else {
         EpiRows<BN, EPI> rows;                    // (no per-row data)
         epi_vec_tile<BN, EPI>(g, nullptr, stg + (warp - 2) * (32 * 68), acc, m0, n0, quarter, ch, lane, rows);
       }
@@ -1170,11 +1231,12 @@ static int launch_persist(const GemmDesc& g, int* d_err, int num_sms, cudaStream
   return -1;
 }
 
+// the pair's kernel for one epilogue
 template <int BN, int STAGES, int EPI>
 static int launch_pair_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s) {
   const int tiles = ceil_div(g.N, BN) * ceil_div(g.M, 2 * kBM);
   const size_t smem = (size_t)STAGES * (kBM * kBK * 2 + BN / 2 * kBK * 2) +
-                      (EPI == EPI_HEAD ? 0 : kEpiWarps * 32 * 68 * 4) + 1024 + 256;
+                      (EPI == EPI_LOGITS ? kEpiWarps * 32 * 68 * 4 : 0) + 1024 + 256;
   static PerDevice attr;
   set_smem_attr(attr, k_gemm_tc_pair<BN, STAGES, EPI>, smem);
   CUtensorMap ma, mw;
@@ -1195,6 +1257,17 @@ static int launch_pair_epi(const GemmDesc& g, int* d_err, int num_sms, cudaStrea
   cfg.attrs = at;
   cfg.numAttrs = g_pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k_gemm_tc_pair<BN, STAGES, EPI>, ma, mw, a) == cudaSuccess ? 0 : -1;
+}
+
+// the row epilogues store (and load) whole 32-byte sectors: rows of 64-column
+// blocks at 32-byte aligned addresses
+static bool pair_rows_ok(const GemmDesc& g) {
+  const Epi& e = g.epi;
+  if (g.N % 64) return false;
+  if (e.kind == EPI_STORE_F32) return !(reinterpret_cast<uintptr_t>(e.outf) & 31) && e.ldo % 8 == 0;
+  if (e.kind == EPI_BIAS_GELU)
+    return !(reinterpret_cast<uintptr_t>(e.out) & 31) && e.ldo % 16 == 0 && !(reinterpret_cast<uintptr_t>(e.bias) & 15);
+  return false;
 }
 
 template <int BN, int STAGES, int AT>
@@ -1242,19 +1315,27 @@ static int active_clusters(int cs) {
 int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   const int num_sms = device_sms();
   const bool persist = !(g_gemm_flags & kGemmNoPersist);
-  // CTA pairs where their rounds of 256 x 256 tiles are many and deep enough
-  // to outweigh the pair's start (about 4 us) and its coarser rounds; one-CTA
-  // loop -> pairs, microseconds: records 2048 x 50,257 at K = 1024 162 -> 146,
-  // K = 768 147 -> 134, 1024 x 50,257 x 768 (11 rounds) 74.3 -> 71.5, 512 x
-  // 50,257 x 1024 (6) 57.3 -> 52.7; but 1024 x 30,522 x 768 (7) 47.6 -> 51.5,
-  // 2100 x 50,257 x 256 82 -> 99; logits 2048 x 50,257 197 -> 179; fp32
-  // products 4096 x 4096 x 1024 (4) 39.0 -> 37.0, 4096 x 3072 x 768 (3) 25.3 -> 26.0
-  const long long depth = (long long)ceil_div(ceil_div(g.N, 256) * ceil_div(g.M, 2 * kBM), num_sms / 2) * g.K;
-  if (persist && ceil_div(g.N, 256) * ceil_div(g.M, kBM) > num_sms && num_sms >= 2 &&   // (no split-K below either)
-      (depth >= 6144 || (g.K >= 1024 && depth >= 4096))) {
-    if (g.epi.kind == EPI_HEAD) return launch_pair_epi<256, 6, EPI_HEAD>(g, d_err, num_sms, s);
-    if (g.epi.kind == EPI_LOGITS) return launch_pair_epi<256, 4, EPI_LOGITS>(g, d_err, num_sms, s);
-    if (g.epi.kind == EPI_STORE_F32) return launch_pair_epi<256, 4, EPI_STORE_F32>(g, d_err, num_sms, s);
+  // CTA pairs past a wave of one-CTA tiles (those never split K), where their
+  // rounds of 256 x 256 tiles are many and deep enough to outweigh the pair's
+  // start (about 4 us) and its coarser rounds.  One-CTA loop -> pairs,
+  // microseconds.  Row epilogues, from three rounds: MLP-up 4096 x 3072 x 768 in
+  // a step 28.4 -> 26.0, 4096 x 4096 x 1024 37.3 -> 35.4; fp32 products 4096 x
+  // 3072 x 768 26.5 -> 24.7, 4096 x 4096 x 1024 39.0 -> 32.8, 8192 x 4096 x 4096
+  // 190 -> 153 (1.80 PFLOP/s); at two rounds 2560 x 3072 x 768 15.8 -> 16.9.
+  // Records and logits: 2048 x 50,257 at K = 1024 162 -> 146, K = 768 147 -> 134,
+  // 1024 x 50,257 x 768 (11 rounds) 74.3 -> 71.5, 512 x 50,257 x 1024 (6) 57.3 ->
+  // 52.7; but 1024 x 30,522 x 768 (7) 47.6 -> 51.5, 2100 x 50,257 x 256 82 -> 99;
+  // logits 2048 x 50,257 197 -> 179.
+  if (persist && ceil_div(g.N, 256) * ceil_div(g.M, kBM) > num_sms && num_sms >= 2) {
+    const int rounds = ceil_div(ceil_div(g.N, 256) * ceil_div(g.M, 2 * kBM), num_sms / 2);
+    const long long depth = (long long)rounds * g.K;
+    const bool deep = depth >= 6144 || (g.K >= 1024 && depth >= 4096);
+    if (g.epi.kind == EPI_HEAD && deep) return launch_pair_epi<256, 6, EPI_HEAD>(g, d_err, num_sms, s);
+    if (g.epi.kind == EPI_LOGITS && deep) return launch_pair_epi<256, 4, EPI_LOGITS>(g, d_err, num_sms, s);
+    if (pair_rows_ok(g) && g.K >= 768 && (rounds >= 3 || deep)) {
+      if (g.epi.kind == EPI_STORE_F32) return launch_pair_epi<256, 6, EPI_STORE_F32>(g, d_err, num_sms, s);
+      if (g.epi.kind == EPI_BIAS_GELU) return launch_pair_epi<256, 6, EPI_BIAS_GELU>(g, d_err, num_sms, s);
+    }
   }
   // LM-head records: 256-wide tiles
   if (g.epi.kind == EPI_HEAD) {

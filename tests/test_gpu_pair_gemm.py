@@ -16,7 +16,9 @@ pytestmark = pytest.mark.gpu
     (2100, 2340, 3072),     # ragged in both; the second CTA's last tile is empty (rows 2100 .. past 2176)
     (4500, 1028, 4096),     # 20 rows in the last pair's second CTA, 4 columns in the last tile
     (19500, 64, 3072),      # one narrow column tile, 77 pairs of row tiles on 76 CTA pairs
-    (4096, 4096, 1024),     # full tiles, four rounds
+    (4096, 4096, 1024),     # full tiles, four rounds; row epilogue
+    (4100, 3008, 768),      # row epilogue: four rows in the last pair, a tile of three 64-column blocks
+    (4100, 3012, 768),      # N not a multiple of 64: the one-CTA loop
 ])
 def test_pair_gemm_matches_fp64_matmul(env, M, N, K):  # noqa: F811
     torch, lib = env
