@@ -516,7 +516,11 @@ k_attention_mma(const __grid_constant__ CUtensorMap map_kv, AttnArgs a) {
 template <int NBUF, bool TWO>
 static int launch_nb(const CUtensorMap& map, const AttnArgs& a, int n_groups, cudaStream_t s) {
   static PerDevice attr;
-  const size_t smem = smem_bytes(NBUF, a.pg_cap);
+  // fewer CTAs than SMs: at most two per SM, so that dependent launch spreads
+  // them (as the skinny projections; one sequence 595 -> 592 us per two calls,
+  // eight 851 -> 845)
+  size_t smem = smem_bytes(NBUF, a.pg_cap);
+  if ((long)n_groups * a.H * a.n_split <= device_sms()) smem = std::max(smem, (size_t)76 * 1024);
   set_smem_attr(attr, k_attention_mma<NBUF, TWO>, smem);
   if (!a.cluster_merge) {
     kf_launch(k_attention_mma<NBUF, TWO>, dim3(n_groups, a.H, a.n_split), dim3(kThr), smem, s, map, a);

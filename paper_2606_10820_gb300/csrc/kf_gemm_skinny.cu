@@ -34,6 +34,8 @@
 // flags kErrTimeout and stores nothing.
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "kf_mma.cuh"
 #include "kf_tc.cuh"
 
@@ -440,7 +442,13 @@ template <int EPI>
 static int launch_skinny_epi(const GemmDesc& g, int* d_err, cudaStream_t s) {
   int splits, kc, m_pad;
   skinny_plan(g, &splits, &kc, &m_pad);
-  const size_t smem = skinny_smem(kc, m_pad);
+  // At most three CTAs per SM.  Launched dependently, while the kernel before
+  // holds one CTA on most SMs, smaller CTAs piled up on the few SMs that it left
+  // free (five or six each) and the kernel ended with those: padding from 36 KB
+  // took two calls of one sequence at k = 4 from 625 to 595 us, of two sequences
+  // 751 -> 714, the AR step of 16 785 -> 748; 50 KB helps one sequence only, 112 KB
+  // delays the CTAs past the first of an SM (the AR step of 16: 768)
+  const size_t smem = std::max(skinny_smem(kc, m_pad), (size_t)74 * 1024);
   if (smem > 200 * 1024) return -1;
   static PerDevice attr;
   set_smem_attr(attr, k_gemm_skinny<EPI>, smem);
