@@ -5,27 +5,26 @@
 // is a stream of W with M FMAs per weight: at 64 rows the FMA pipes (about
 // 37 TFMA/s) take as long as HBM, below that HBM and the launch chain do.
 // Tile and split, and why:
-//  - a CTA covers 16 RG rows x 64 columns; a warp 16 rows x 64 columns, each
-//    lane two columns.  All lanes of a warp share their rows, so the A reads
-//    are broadcasts (one shared-memory wavefront) and only the two W reads
-//    per four k take four: 24 wavefronts against 64 FFMA2, where square
-//    8 x 8 thread tiles would take 64 and be bound by shared memory;
+//  - a CTA covers 16 RG rows x 64 columns, a warp 16 rows x 64 columns, a lane 8
+//    rows x 4 columns (half a warp shares its rows): 12 16-byte shared-memory reads
+//    per 64 FFMA2.  Each read takes four cycles of the 128 B/clk that shared memory
+//    returns, broadcast or not: 16 rows x 2 columns per lane needed 18;
 //  - FFMA2 pairs run along k (even and odd k in the two halves), the order in
 //    which both operands lie in memory: no transpose, and two shorter sums;
 //  - the KG warps that share a row group each take their part of every
-//    64-wide K stage, and K is split over a cluster of up to 8 CTAs while the
-//    tiles leave SMs idle; partials meet in shared memory (DSMEM across the
+//    64-wide K stage, and K is split over a cluster of up to 8 CTAs while every
+//    cluster runs at once; partials meet in shared memory (DSMEM across the
 //    cluster) in a fixed order: deterministic, no workspace, no atomics;
-//  - three cp.async stages; the first stages' W rows are read before the
+//  - four cp.async stages; the first stages' W rows are read before the
 //    dependency wait (weights do not change during a step).
 // Measured at 64 rows, per launch with its launch latency (about 5 us),
 // before -> now (before: 32 x 128 tiles, one row per lane, no K split, 12 to
-// 48 CTAs): 2304 x 768 170 -> 17 us, 768 x 768 159 -> 15, 3072 x 768 163 ->
-// 26, 768 x 3072 613 -> 24, head 30,522 x 768 (32 rows) 195 -> 67; a decode
-// call of the 768-wide 12-layer model, 8 sequences at k = 4, 14.3 -> 1.05 ms.
-// The FMA pipes are 20-40 % busy; the rest is the first loads, the cluster
-// barriers and the reduction.  Sixteen warps per CTA (twice the K groups)
-// measured slower: 3072 x 768 26 -> 34 us (twice the partials to sum).
+// 48 CTAs): 2304 x 768 170 -> 16 us, 768 x 768 159 -> 14, 3072 x 768 163 ->
+// 21, 768 x 3072 613 -> 22, head 30,522 x 768 (32 rows) 195 -> 60; two decode calls
+// of the 768-wide 12-layer model, 8 sequences at k = 4, and their logits 29.6
+// -> 1.72 ms.  What is left is the first loads, the cluster barriers and the
+// reduction.  Sixteen warps per CTA (twice the K groups) measured slower (1.92 ms:
+// twice the partials to sum), plain FFMA as well (1.77 ms: issue slots).
 #include <algorithm>
 
 #include "kf_tc.cuh"
@@ -36,7 +35,7 @@ namespace {
 constexpr int kFN = 64;              // columns per CTA
 constexpr int kFK = 64;              // K per stage
 constexpr int kFLd = kFK + 4;        // floats per row: lanes 4 banks apart, conflict-free 16-byte reads
-constexpr int kFStages = 3;
+constexpr int kFStages = 4;
 
 __host__ __device__ constexpr int f32_kg(int RG) { return RG == 1 ? 8 : RG == 2 ? 4 : 2; }
 __host__ __device__ constexpr int f32_stage_floats(int RG) { return (16 * RG + kFN) * kFLd; }
@@ -45,13 +44,10 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool i
   const int n = in ? 16 : 0;         // 0: zero-fill, src not read
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
-__device__ __forceinline__ unsigned long long ffma2(unsigned long long a, unsigned long long b,
-                                                    unsigned long long c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
+// acc += {a0 w0, a1 w1}
+__device__ __forceinline__ void fma2(float2& acc, float a0, float a1, float w0, float w1) {
+  acc = f2_split(fma_f2(f2(a0, a1), f2(w0, w1), f2(acc.x, acc.y)));
 }
-
 // four consecutive columns of one row
 __device__ __forceinline__ void epi_f32_vec4(const Epi& e, int row, int col, float4 v, int N) {
   switch (e.kind) {
@@ -81,17 +77,27 @@ __global__ void __launch_bounds__(RG * f32_kg(RG) * 32) k_gemm_f32(GemmDesc g, i
   const float* W = static_cast<const float*>(g.W);
   const uint32_t sbase = smem_u32(fsm);
 
-  auto load = [&](int i, const float* src, int ld, int first, int n_rows, int limit, int at) {
-    const uint32_t dst = sbase + (uint32_t)((i % kFStages) * SF + at * kFLd) * 4;
-    const int kb = k0 + i * kFK;
-    for (int c = t; c < n_rows * (kFK / 4); c += NT) {
-      const int r = c / (kFK / 4), k = kb + (c % (kFK / 4)) * 4;
-      const bool in = first + r < limit && k < k1;
-      cp_async16(dst + (uint32_t)(r * kFLd + (c % (kFK / 4)) * 4) * 4, in ? src + (size_t)(first + r) * ld + k : src, in);
+  // stage i: each thread copies the same 16-byte column of every NT / 16-th row
+  constexpr int kC = kFK / 4, kStep = NT / kC;        // 16-byte columns, rows per pass
+  const int lr = t / kC, lk = (t % kC) * 4;
+  const uint32_t ldst = sbase + (uint32_t)(lr * kFLd + lk) * 4;
+  auto load = [&](int i, const float* src, int ld, int rows, int limit, int at) {
+    const uint32_t dst = ldst + (uint32_t)((i % kFStages) * SF + at * kFLd) * 4;
+    const int k = i * kFK;
+    const bool ink = k0 + lk + k < k1;
+    src += k;
+#pragma unroll
+    for (int r = 0; r < rows; r += kStep) {
+      if (rows % kStep && r + lr >= rows) break;
+      const bool in = ink && r + lr < limit;
+      cp_async16(dst + (uint32_t)(r * kFLd) * 4, in ? src : g.W, in);
+      src += (size_t)kStep * ld;
     }
   };
-  auto load_w = [&](int i) { load(i, W, g.ldw, col0, kFN, g.N, BM); };
-  auto load_a = [&](int i) { load(i, A, g.lda, row0, BM, g.M, 0); };
+  const float* wsrc = W + (size_t)(col0 + lr) * g.ldw + k0 + lk;    // (not read past N, M or k1)
+  const float* asrc = A + (size_t)(row0 + lr) * g.lda + k0 + lk;
+  auto load_w = [&](int i) { load(i, wsrc, g.ldw, kFN, g.N - col0, BM); };
+  auto load_a = [&](int i) { load(i, asrc, g.lda, BM, g.M - row0, 0); };
   auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
 
   // weights are constant during a step: read ahead of the dependency
@@ -103,9 +109,15 @@ __global__ void __launch_bounds__(RG * f32_kg(RG) * 32) k_gemm_f32(GemmDesc g, i
     commit();                                        // the first group holds the W rows above too
   }
 
-  unsigned long long acc[16][2];
+  // lanes 0..15 take the warp's first 8 rows, lanes 16..31 the other 8; a lane
+  // has columns l, l + 16, l + 32, l + 48
+  constexpr int R = 8, C = 4;
+  const int half = lane >> 4, l16 = lane & 15;
+  float2 acc[R][C];                                  // even k, odd k
 #pragma unroll
-  for (int r = 0; r < 16; ++r) acc[r][0] = acc[r][1] = 0ull;
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[r][c] = make_float2(0.f, 0.f);
   for (int i = 0; i < nst; ++i) {
     asm volatile("cp.async.wait_group %0;" ::"n"(kFStages - 2) : "memory");
     __syncthreads();                                 // stage i is here; stage i - 1 has been read
@@ -114,49 +126,50 @@ __global__ void __launch_bounds__(RG * f32_kg(RG) * 32) k_gemm_f32(GemmDesc g, i
       load_a(i + kFStages - 1);
     }
     commit();
-    const float* as = fsm + (i % kFStages) * SF + (rg * 16) * kFLd + kg * KW;
-    const float* ws = fsm + (i % kFStages) * SF + (BM + lane) * kFLd + kg * KW;
-    // four rows' A reads run ahead of the FMAs of the four before them, and
-    // an accumulator's two FMAs lie eight instructions apart
-    ulonglong2 a[2][4];
+    const float* as = fsm + (i % kFStages) * SF + (rg * 16 + half * R) * kFLd + kg * KW;
+    const float* ws = fsm + (i % kFStages) * SF + (BM + l16) * kFLd + kg * KW;
+    auto ldw = [&](int k, float4* w) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) a[0][r] = *reinterpret_cast<const ulonglong2*>(as + r * kFLd);
-    ulonglong2 w0 = *reinterpret_cast<const ulonglong2*>(ws), w1 = *reinterpret_cast<const ulonglong2*>(ws + 32 * kFLd);
+      for (int c = 0; c < C; ++c) w[c] = *reinterpret_cast<const float4*>(ws + 16 * c * kFLd + k);
+    };
+    // two rows' A reads run ahead of the FMAs of the two before them, and an
+    // accumulator's two FMAs lie eight instructions apart
+    float4 a[2][2], w[C], wn[C];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) a[0][r] = *reinterpret_cast<const float4*>(as + r * kFLd);
+    ldw(0, w);
 #pragma unroll 1
     for (int k = 0; k < KW; k += 4) {
       const int kn = k + 4 < KW ? k + 4 : 0;         // (the last read is not used)
-      const ulonglong2 n0 = *reinterpret_cast<const ulonglong2*>(ws + kn);
-      const ulonglong2 n1 = *reinterpret_cast<const ulonglong2*>(ws + 32 * kFLd + kn);
+      ldw(kn, wn);
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int rn = (b + 1) % 4 * 4;
+      for (int b = 0; b < R / 2; ++b) {
+        const int rn = (b + 1) % (R / 2) * 2;
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-          a[(b + 1) & 1][r] = *reinterpret_cast<const ulonglong2*>(as + (rn + r) * kFLd + (b == 3 ? kn : k));
+        for (int r = 0; r < 2; ++r)
+          a[(b + 1) & 1][r] = *reinterpret_cast<const float4*>(as + (rn + r) * kFLd + (b == R / 2 - 1 ? kn : k));
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          acc[4 * b + r][0] = ffma2(a[b & 1][r].x, w0.x, acc[4 * b + r][0]);
-          acc[4 * b + r][1] = ffma2(a[b & 1][r].x, w1.x, acc[4 * b + r][1]);
-        }
+        for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          acc[4 * b + r][0] = ffma2(a[b & 1][r].y, w0.y, acc[4 * b + r][0]);
-          acc[4 * b + r][1] = ffma2(a[b & 1][r].y, w1.y, acc[4 * b + r][1]);
-        }
+          for (int c = 0; c < C; ++c) fma2(acc[2 * b + r][c], a[b & 1][r].x, a[b & 1][r].y, w[c].x, w[c].y);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int c = 0; c < C; ++c) fma2(acc[2 * b + r][c], a[b & 1][r].z, a[b & 1][r].w, w[c].z, w[c].w);
       }
-      w0 = n0;
-      w1 = n1;
+#pragma unroll
+      for (int c = 0; c < C; ++c) w[c] = wn[c];
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   // partials [KG][BM][kFLd]: even + odd k
-  float* P = fsm + (size_t)(kg * BM + rg * 16) * kFLd;
+  float* P = fsm + (size_t)(kg * BM + rg * 16 + half * R) * kFLd + l16;
 #pragma unroll
-  for (int r = 0; r < 16; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
-      P[r * kFLd + lane + 32 * j] = __uint_as_float((uint32_t)acc[r][j]) + __uint_as_float((uint32_t)(acc[r][j] >> 32));
+    for (int c = 0; c < C; ++c)
+      P[r * kFLd + 16 * c] = acc[r][c].x + acc[r][c].y;
   if (splits > 1) cluster_sync();
   else __syncthreads();
   // CTA q of the cluster sums rows q, q + S, ...: splits in order, then warps
@@ -195,16 +208,25 @@ __global__ void __launch_bounds__(RG * f32_kg(RG) * 32) k_gemm_f32(GemmDesc g, i
 template <int RG>
 static int launch_rg(const GemmDesc& g, cudaStream_t s) {
   constexpr int KG = f32_kg(RG);
-  const size_t smem = (size_t)kFStages * f32_stage_floats(RG) * 4;
-  static PerDevice attr;
-  set_smem_attr(attr, k_gemm_f32<RG>, smem);
   const int n_tiles = ceil_div(g.N, kFN), m_tiles = ceil_div(g.M, 16 * RG);
   const int st = ceil_div(g.K, kFK);
-  // K over a cluster of up to 8 CTAs while they fit in one wave of one CTA
-  // per SM, one stage each at least
-  int splits = std::max(1, std::min({8, st, device_sms() / std::max(1, n_tiles * m_tiles)}));
+  // K over a cluster of up to 8 CTAs, one stage each at least, while all
+  // clusters run at once with an SM per CTA (a cluster lies within a GPC: 48 of 3
+  // do not fit 152 SMs, and the last two doubled up on their SMs: 3072 x 768 at 64
+  // rows 24 us at 3 splits, 16 at 2)
+  int splits = std::min(8, st);
+  while (splits > 1 && n_tiles * m_tiles > active_clusters(splits)) --splits;
   const int kps = ceil_div(st, splits) * kFK;
   splits = ceil_div(g.K, kps);                       // no empty splits
+  // within a wave an SM per CTA (more than half of its shared memory): two on one
+  // SM leave another idle, and dependent launch makes that common, the next
+  // kernel's CTAs arriving while some SMs are still busy (a step 2.14 -> 1.79 ms
+  // for two calls); past a wave two per SM hide each other's loads
+  const size_t need = (size_t)kFStages * f32_stage_floats(RG) * 4;
+  const bool alone = n_tiles * m_tiles * splits <= device_sms();
+  const size_t smem = alone ? std::max(need, (size_t)116 * 1024) : need;
+  static PerDevice attr;
+  set_smem_attr(attr, k_gemm_f32<RG>, smem);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_tiles, m_tiles, splits);
   cfg.blockDim = dim3(RG * KG * 32);

@@ -1288,7 +1288,7 @@ static int launch_bn(const GemmDesc& g, int* d_err, int num_sms, cudaStream_t s,
 // CTA per SM (every k_gemm_tc takes more than half of an SM's shared memory): a
 // cluster lies within a GPC, so fewer than num_sms / cs (152 SMs: 76, 36 and 15
 // clusters of 2, 4 and 8)
-static int active_clusters(int cs) {
+int active_clusters(int cs) {
   static PerDevice pd[9];
   return (int)per_device(pd[cs], [&] {
     constexpr size_t smem = (size_t)4 * 2 * (kBM * kBK * 2 + 64 * kBK * 2) + 1024 + 256 + sizeof(EpiMeta);

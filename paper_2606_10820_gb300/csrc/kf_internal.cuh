@@ -458,6 +458,9 @@ int launch_gemm_f32(const GemmDesc& g, cudaStream_t s);
 bool tc_gemm_supported(const GemmDesc& g);
 int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s);
 
+// clusters of cs <= 8 CTAs that run at the same time at one CTA per SM
+int active_clusters(int cs);
+
 // Skinny projections (kf_gemm_skinny.cu): M <= 64 rows on warp-level MMA,
 // weights staged before the dependency wait.  The fused RMSNorm scale comes
 // from the A rows themselves (epi.ss_in set means "normed input"; it is not
