@@ -468,6 +468,13 @@ static int upload_page_row(kf_ctx* c, int b) {
   return KF_OK;
 }
 
+// The most rows of a prefill's last chunk: a remainder of up to a quarter of a
+// chunk joins it, because a chunk of few rows is a chain of five launches per
+// layer that leaves the chip idle (768-wide, 12 layers, microseconds per prefill
+// with the remainder apart -> joined: 5 prompts of 1000 2380 -> 1821, 16 of 539
+// 3289 -> 2889).
+static int last_chunk_rows(const kf_ctx* c) { return c->prefill_rows + c->prefill_rows / 4; }
+
 // ------------------------------------------------------------- C ABI
 extern "C" {
 
@@ -662,7 +669,7 @@ int kf_init(const kf_config* cfg_in, const kf_weights* w, void* stream, kf_ctx**
   c->pend_stride = MK;
   c->NR_cap = round_up(MB * MK, 128);
   c->prefill_rows = round_up(cfg.prefill_rows, 128);
-  c->R_cap = std::max(round_up(MB * 2 * MK, 128), c->prefill_rows);
+  c->R_cap = std::max(round_up(MB * 2 * MK, 128), round_up(last_chunk_rows(c), 128));
   const int R = c->R_cap;
   if ((r = dalloc(c, &c->d_len, MB * 4)) || (r = dalloc(c, &c->d_len0, MB * 4)) ||
       (r = dalloc(c, &c->d_order, MB * 4)) ||
@@ -697,9 +704,9 @@ int kf_init(const kf_config* cfg_in, const kf_weights* w, void* stream, kf_ctx**
 }
 
 // Prefill: the KV of each listed slot's first n tokens (positions 0..n-1),
-// in row chunks of up to prefill_rows, attention groups of consecutive rows of a
-// sequence: up to 128 for the tcgen05 kernel, else up to 16.  The slots' pages
-// must be allocated and uploaded.
+// in row chunks of prefill_rows (the last one up to last_chunk_rows), attention
+// groups of consecutive rows of a sequence: up to 128 for the tcgen05 kernel,
+// else up to 16.  The slots' pages must be allocated and uploaded.
 // The rows of a chunk's attention groups: 128 (tcgen05) once the 128-row items
 // cover the SMs and hold 40 rows or more on average, else 16 (warp-level MMA, which
 // also splits the keys of few long rows).  Measured, 768-wide model, 4 layers,
@@ -752,11 +759,19 @@ static int prefill_rows(kf_ctx* c, const std::vector<PrefillSeq>& seqs) {
     r_tok.clear(); r_seq.clear(); r_pos.clear(); runs.clear(); grp.clear();
     return KF_OK;
   };
+  long long left = 0;              // rows not yet in a flushed chunk
+  for (const PrefillSeq& q : seqs) left += q.n;
+  auto chunk_rows = [&] { return left <= last_chunk_rows(c) ? (int)left : c->prefill_rows; };
+  int cap = chunk_rows();
   for (const PrefillSeq& q : seqs) {
     int p = 0;
     while (p < q.n) {
-      if ((int)r_tok.size() == c->prefill_rows) KF_TRY(flush());
-      int take = std::min(q.n - p, c->prefill_rows - (int)r_tok.size());
+      if ((int)r_tok.size() == cap) {
+        KF_TRY(flush());
+        left -= cap;
+        cap = chunk_rows();
+      }
+      int take = std::min(q.n - p, cap - (int)r_tok.size());
       runs.push_back(make_int4(q.slot, (int)r_tok.size(), take, p));
       for (int i = 0; i < take; ++i) {
         r_tok.push_back(q.tok[p + i]);
