@@ -361,6 +361,12 @@ void launch_rope_append(bool bf16, int R, const void* qkv, int d, int H, int hd,
 // If rounding leaves no crossing, the largest id with exp(l - M) > 0 wins.
 // ARGMAX: the lowest id attaining M.
 constexpr int kSelThreads = 256;
+// bf16: twice the threads per row up to this many rows (the phases between a
+// row's barriers shorten; past it more rows per SM win).  256 -> 512 threads, LM
+// head and selection, microseconds: 1 row 16.5 -> 15.6, 256 rows x 30,522 24 ->
+// 20.8, 512 x 50,257 54.6 -> 50.0; but 1024 rows 77 -> 82, 2048 134 -> 148 (128
+// threads there 140)
+constexpr int kSelWideRows = 512;
 
 __device__ __forceinline__ void ld_vec(const float* p, float* o) {
   float4 a = *reinterpret_cast<const float4*>(p);
@@ -399,8 +405,8 @@ __device__ __forceinline__ void emit_token(int32_t* tokens, int zrow, int tok, c
   }
 }
 
-template <typename TA>
-__global__ void __launch_bounds__(kSelThreads)
+template <typename TA, int NT>
+__global__ void __launch_bounds__(NT)
 k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restrict__ head_in, int d,
               const TA* __restrict__ w_head_all, int V, float inv_tau, int map_kind,
               const float* __restrict__ noise, int32_t* __restrict__ tokens, int mtp_rows,
@@ -432,16 +438,16 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
   using Acc = typename std::conditional<sizeof(TA) == 4, double, float>::type;
   const HeadRec* rec = rec_all + (size_t)row * nchunk;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  __shared__ float s_red[kSelThreads / 32];
-  __shared__ Acc s_acc[kSelThreads / 32];
-  __shared__ int s_redi[kSelThreads / 32];
+  __shared__ float s_red[NT / 32];
+  __shared__ Acc s_acc[NT / 32];
+  __shared__ int s_redi[NT / 32];
   __shared__ float s_M;
   __shared__ Acc s_T;
   __shared__ int s_chunk;
   __shared__ Acc s_before;
 
   // contiguous chunk range per thread keeps id order inside each partial sum
-  const int per = ceil_div(nchunk, kSelThreads);
+  const int per = ceil_div(nchunk, NT);
   const int c0 = min(nchunk, t * per), c1 = min(nchunk, c0 + per);
 
   // 1) M and (for argmax) the lowest id attaining it; the thread's records
@@ -478,7 +484,7 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
   if (t == 0) {
     float M = s_red[0];
     int A = s_redi[0];
-    for (int w = 1; w < kSelThreads / 32; ++w)
+    for (int w = 1; w < NT / 32; ++w)
       if (s_red[w] > M || (s_red[w] == M && s_redi[w] < A)) { M = s_red[w]; A = s_redi[w]; }
     s_M = M;
     s_redi[0] = A;
@@ -514,16 +520,16 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
   if (lane == 0) lane_excl = 0;
   if (lane == 31) s_acc[warp] = inc;
   __syncthreads();
-  __shared__ Acc s_wexcl[kSelThreads / 32 + 1];
+  __shared__ Acc s_wexcl[NT / 32 + 1];
   if (t == 0) {
     Acc run = 0;
-    for (int w = 0; w < kSelThreads / 32; ++w) {
+    for (int w = 0; w < NT / 32; ++w) {
       s_wexcl[w] = run;
       run += s_acc[w];
     }
-    s_wexcl[kSelThreads / 32] = run;     // S
+    s_wexcl[NT / 32] = run;     // S
     s_T = (Acc)noise[zrow] * run;
-    s_redi[2] = kSelThreads;             // first crossing thread (none yet)
+    s_redi[2] = NT;             // first crossing thread (none yet)
   }
   __syncthreads();
   const Acc T = s_T;
@@ -550,7 +556,7 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
     s_before = before;
     s_redi[1] = 0;
   }
-  if (t == 0 && s_redi[2] >= kSelThreads) {
+  if (t == 0 && s_redi[2] >= NT) {
     // no crossing at all (z near 1): the last chunk with mass, last id in it
     int cstar = nchunk - 1;
     while (cstar > 0 && !(rec[cstar].s * expf(rec[cstar].m - M) > 0.f)) --cstar;
@@ -568,7 +574,7 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
     // the warp's NQ ids side by side, so their weight loads are in flight together
     const TA* hr = head_in + (size_t)hrow * d;
     constexpr int VEC = 16 / sizeof(TA);
-    constexpr int NQ = kChunk / (kSelThreads / 32);
+    constexpr int NQ = kChunk / (NT / 32);
     const int jj0 = warp * NQ;
     float acc[NQ];
 #pragma unroll
@@ -624,12 +630,16 @@ void launch_head_select(bool bf16, int n_rows, const HeadRec* rec, int nchunk, c
                         const float* noise, int32_t* tokens, int mtp_rows, size_t head_stride,
                         const int* err, const StepCommit& cm, cudaStream_t s) {
   if (n_rows == 0) return;
-  if (bf16)
-    kf_launch(k_head_select<__nv_bfloat16>, dim3(n_rows), dim3(kSelThreads), 0, s, rec, nchunk,
-        (const __nv_bfloat16*)head_in, d, (const __nv_bfloat16*)w_head, V, inv_tau, map_kind,
-        noise, tokens, mtp_rows, head_stride, err, cm);
+  auto bf = [&](auto kern, int nt) {
+    kf_launch(kern, dim3(n_rows), dim3(nt), 0, s, rec, nchunk, (const __nv_bfloat16*)head_in, d,
+              (const __nv_bfloat16*)w_head, V, inv_tau, map_kind, noise, tokens, mtp_rows, head_stride, err, cm);
+  };
+  if (bf16 && n_rows <= kSelWideRows)
+    bf(k_head_select<__nv_bfloat16, 2 * kSelThreads>, 2 * kSelThreads);
+  else if (bf16)
+    bf(k_head_select<__nv_bfloat16, kSelThreads>, kSelThreads);
   else
-    kf_launch(k_head_select<float>, dim3(n_rows), dim3(kSelThreads), 0, s, rec, nchunk, (const float*)head_in, d,
+    kf_launch(k_head_select<float, kSelThreads>, dim3(n_rows), dim3(kSelThreads), 0, s, rec, nchunk, (const float*)head_in, d,
         (const float*)w_head, V, inv_tau, map_kind, noise, tokens, mtp_rows, head_stride, err, cm);
 }
 

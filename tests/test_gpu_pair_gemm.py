@@ -38,7 +38,8 @@ def test_pair_gemm_matches_fp64_matmul(env, M, N, K):  # noqa: F811
 # (400 x 25,000 x 3072: the records on CTA pairs, a ragged second row pair;
 # vocabularies that end inside a chunk, at one id, on a chunk; fewer than a
 # wave of row tiles; argmax ties within and across chunks below)
-@pytest.mark.parametrize("rows,V,d", [(400, 25000, 3072), (129, 33, 64), (7, 1, 64), (300, 992, 128), (2048, 1000, 128)])
+@pytest.mark.parametrize("rows,V,d", [(400, 25000, 3072), (129, 33, 64), (7, 1, 64), (300, 992, 128), (2048, 1000, 128),
+                                      (512, 70, 64), (513, 70, 64)])     # 512 and 256 threads per row
 @pytest.mark.parametrize("map_kind", [0, 1])
 def test_head_records_at_edges(head_env, rows, V, d, map_kind):  # noqa: F811
     torch, lib = head_env
