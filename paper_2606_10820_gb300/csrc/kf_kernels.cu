@@ -363,10 +363,20 @@ void launch_rope_append(bool bf16, int R, const void* qkv, int d, int H, int hd,
 constexpr int kSelThreads = 256;
 // bf16: twice the threads per row up to this many rows (the phases between a
 // row's barriers shorten; past it more rows per SM win).  256 -> 512 threads, LM
-// head and selection, microseconds: 1 row 16.5 -> 15.6, 256 rows x 30,522 24 ->
-// 20.8, 512 x 50,257 54.6 -> 50.0; but 1024 rows 77 -> 82, 2048 134 -> 148 (128
-// threads there 140)
+// head and selection, microseconds: 256 rows x 30,522 23 -> 20.8, 512 x 50,257
+// 53 -> 47.6; but 1024 rows 70 -> 86, 2048 124 -> 162
 constexpr int kSelWideRows = 512;
+// What bounds the kernel at many rows is the chain inside a row (records, maximum,
+// sums, crossing, the chunk's 32 weight rows) times the waves of rows.  Against one
+// thread combining the warps' values between two barriers (7 barriers a row) and
+// records read in place by 32-bit loads, LM head and selection went: 2048 rows x
+// 50,257 icdf 134 -> 124.5 us, argmax 124 -> 114, 1024 rows 77 -> 70, 512 rows
+// 50 -> 47.6, 1 row 15.5 -> 14.7; without the staged copy 2048 rows take 129.6.
+// 64 registers (1024 threads per SM) keep a row's loads in flight together: 1280
+// threads per SM 127.5, 1536 128.3, 768 124.3
+constexpr int kSelThreadsPerSm = 1024;
+constexpr int kSelKeep = 8;               // records a thread holds in registers
+constexpr int kSelStageMax = 40 * 1024;   // bytes of a row's records staged in shared memory (no opt-in size)
 
 __device__ __forceinline__ void ld_vec(const float* p, float* o) {
   float4 a = *reinterpret_cast<const float4*>(p);
@@ -406,11 +416,11 @@ __device__ __forceinline__ void emit_token(int32_t* tokens, int zrow, int tok, c
 }
 
 template <typename TA, int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, kSelThreadsPerSm / NT)
 k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restrict__ head_in, int d,
               const TA* __restrict__ w_head_all, int V, float inv_tau, int map_kind,
               const float* __restrict__ noise, int32_t* __restrict__ tokens, int mtp_rows,
-              size_t head_stride, const int* __restrict__ err, StepCommit cm) {
+              size_t head_stride, const int* __restrict__ err, StepCommit cm, int staged) {
   pdl_wait();
   // one block per mapped row; MTP (mtp_rows = B > 0): block j B + b is head j
   // of sequence b (records in that order), hidden row b, weights w_head + j
@@ -436,42 +446,57 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
   // rounding far above fp32's); fp64 for the fp32 model, so its decision is
   // limited by its fp32 logits and not by ~5e4 fp32 additions
   using Acc = typename std::conditional<sizeof(TA) == 4, double, float>::type;
+  constexpr int NW = NT / 32;
   const HeadRec* rec = rec_all + (size_t)row * nchunk;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  __shared__ float s_red[NT / 32];
-  __shared__ Acc s_acc[NT / 32];
-  __shared__ int s_redi[NT / 32];
-  __shared__ float s_M;
-  __shared__ Acc s_T;
-  __shared__ int s_chunk;
-  __shared__ Acc s_before;
+  __shared__ __align__(16) float s_max[NW];
+  __shared__ __align__(16) int s_arg[NW];
+  __shared__ __align__(16) Acc s_acc[NW];
+  __shared__ __align__(16) Acc s_before[NW];
+  __shared__ __align__(16) int s_chunk[NW];
+  extern __shared__ __align__(16) unsigned char s_stage[];
+  auto rec_at = [](const HeadRec* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
 
-  // contiguous chunk range per thread keeps id order inside each partial sum
+  // contiguous chunk range per thread keeps id order inside each partial sum.
+  // A staged row is copied to shared memory first, 16 bytes a thread side by
+  // side: read in place, each of a warp's loads touches a line per lane (the
+  // ranges lie ~100 bytes apart)
   const int per = ceil_div(nchunk, NT);
   const int c0 = min(nchunk, t * per), c1 = min(nchunk, c0 + per);
+  float z = 0.f;
+  if (map_kind != KF_MAP_ARGMAX) z = noise[zrow];
+  if (staged) {
+    for (int c = t; c < nchunk; c += NT)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(s_stage + (size_t)c * sizeof(HeadRec))),
+                   "l"(rec + c)
+                   : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+  }
 
   // 1) M and (for argmax) the lowest id attaining it; the thread's records
   //    stay in registers for step 2 when they fit
-  constexpr int kKeep = 8;
-  const bool keep = c1 - c0 <= kKeep;
-  float km[kKeep], ks[kKeep];
+  const bool keep = per <= kSelKeep;
+  Acc km[kSelKeep];    // a record's maximum, then its scale exp(m - M)
+  float ks[kSelKeep];
   float m = -INFINITY;
   int am = 0x7fffffff;
 #pragma unroll
-  for (int i = 0; i < kKeep; ++i) {
+  for (int i = 0; i < kSelKeep; ++i) {
     km[i] = -INFINITY;
     ks[i] = 0.f;
     if (keep && c0 + i < c1) {
-      const HeadRec r = rec[c0 + i];
-      km[i] = r.m;
-      ks[i] = r.s;
-      if (r.m > m) { m = r.m; am = r.a; }
+      const float4 r = staged ? reinterpret_cast<const float4*>(s_stage)[c0 + i] : rec_at(rec + c0 + i);
+      km[i] = r.x;
+      ks[i] = r.y;
+      if (r.x > m) { m = r.x; am = __float_as_int(r.z); }
     }
   }
   if (!keep) {
     for (int c = c0; c < c1; ++c) {
-      HeadRec r = rec[c];
-      if (r.m > m) { m = r.m; am = r.a; }
+      const float4 r = rec_at(rec + c);
+      if (r.x > m) { m = r.x; am = __float_as_int(r.z); }
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -479,22 +504,22 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
     int a2 = __shfl_xor_sync(0xffffffffu, am, o);
     if (m2 > m || (m2 == m && a2 < am)) { m = m2; am = a2; }
   }
-  if (lane == 0) { s_red[warp] = m; s_redi[warp] = am; }
+  if (lane == 0) { s_max[warp] = m; s_arg[warp] = am; }
   __syncthreads();
-  if (t == 0) {
-    float M = s_red[0];
-    int A = s_redi[0];
-    for (int w = 1; w < NT / 32; ++w)
-      if (s_red[w] > M || (s_red[w] == M && s_redi[w] < A)) { M = s_red[w]; A = s_redi[w]; }
-    s_M = M;
-    s_redi[0] = A;
+  // every warp combines the warps' values itself: no second barrier for one
+  // thread's answer (nor for the sums, added in warp order, and the crossing)
+  float M = s_max[lane % NW];
+  int A = s_arg[lane % NW];
+#pragma unroll
+  for (int o = NW / 2; o > 0; o >>= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, M, o);
+    const int a2 = __shfl_xor_sync(0xffffffffu, A, o);
+    if (m2 > M || (m2 == M && a2 < A)) { M = m2; A = a2; }
   }
-  __syncthreads();
   if (map_kind == KF_MAP_ARGMAX) {
-    if (t == 0) emit_token(tokens, zrow, s_redi[0], cm);
+    if (t == 0) emit_token(tokens, zrow, A, cm);
     return;
   }
-  const float M = s_M;
 
   // 2) per-thread partial sums (id order inside each range), then a
   //    fixed-order block scan over the threads: lanes by shuffles, warps by
@@ -503,12 +528,15 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
   Acc part = 0;
   if (keep) {
 #pragma unroll
-    for (int i = 0; i < kKeep; ++i)
-      if (c0 + i < c1) part += (Acc)ks[i] * chunk_scale<Acc>(km[i], M);
+    for (int i = 0; i < kSelKeep; ++i)
+      if (c0 + i < c1) {
+        km[i] = chunk_scale<Acc>((float)km[i], M);
+        part += (Acc)ks[i] * km[i];
+      }
   } else {
     for (int c = c0; c < c1; ++c) {
-      HeadRec r = rec[c];
-      part += (Acc)r.s * chunk_scale<Acc>(r.m, M);
+      const float4 r = rec_at(rec + c);
+      part += (Acc)r.y * chunk_scale<Acc>(r.x, M);
     }
   }
   Acc inc = part;
@@ -520,56 +548,56 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
   if (lane == 0) lane_excl = 0;
   if (lane == 31) s_acc[warp] = inc;
   __syncthreads();
-  __shared__ Acc s_wexcl[NT / 32 + 1];
-  if (t == 0) {
-    Acc run = 0;
-    for (int w = 0; w < NT / 32; ++w) {
-      s_wexcl[w] = run;
-      run += s_acc[w];
-    }
-    s_wexcl[NT / 32] = run;     // S
-    s_T = (Acc)noise[zrow] * run;
-    s_redi[2] = NT;             // first crossing thread (none yet)
+  Acc run = 0, wexcl = 0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    if (w == warp) wexcl = run;
+    run += s_acc[w];
   }
-  __syncthreads();
-  const Acc T = s_T;
-  const Acc excl = s_wexcl[warp] + lane_excl, incl = s_wexcl[warp] + inc;
-  {
-    const unsigned cross = __ballot_sync(0xffffffffu, incl > T);
-    if (lane == 0 && cross) atomicMin(&s_redi[2], warp * 32 + __ffs(cross) - 1);
-  }
-  __syncthreads();
-  if (t == s_redi[2]) {
-    // the crossing range: walk its chunks in id order from its exclusive prefix
-    Acc acc = excl;
+  const Acc T = (Acc)z * run;   // run: S
+  const Acc excl = wexcl + lane_excl, incl = wexcl + inc;
+  const unsigned cross = __ballot_sync(0xffffffffu, incl > T);
+  // the first crossing lane of each warp walks its range's chunks in id order
+  // from its exclusive prefix; the first such warp's answer is the row's
+  if (lane == (cross ? __ffs(cross) - 1 : 0)) {
+    Acc acc = excl, before = excl;
     int cstar = c1 - 1;
-    Acc before = acc;
-    for (int c = c0; c < c1; ++c) {
-      HeadRec r = rec[c];
-      const Acc sc = (Acc)r.s * chunk_scale<Acc>(r.m, M);
-      // the range's own order can round differently from its partial sum:
-      // its last chunk takes the crossing then
-      if (acc + sc > T || c == c1 - 1) { cstar = c; before = acc; break; }
-      acc += sc;
+    bool found = false;
+    if (keep) {
+#pragma unroll
+      for (int i = 0; i < kSelKeep; ++i)
+        if (!found && c0 + i < c1) {
+          const Acc sc = (Acc)ks[i] * km[i];
+          // the range's own order can round differently from its partial sum:
+          // its last chunk takes the crossing then
+          if (acc + sc > T || c0 + i == c1 - 1) { cstar = c0 + i; before = acc; found = true; }
+          acc += sc;
+        }
+    } else if (cross) {
+      for (int c = c0; c < c1; ++c) {
+        const float4 r = rec_at(rec + c);
+        const Acc sc = (Acc)r.y * chunk_scale<Acc>(r.x, M);
+        if (acc + sc > T || c == c1 - 1) { cstar = c; before = acc; break; }
+        acc += sc;
+      }
     }
-    s_chunk = cstar;
-    s_before = before;
-    s_redi[1] = 0;
-  }
-  if (t == 0 && s_redi[2] >= NT) {
-    // no crossing at all (z near 1): the last chunk with mass, last id in it
-    int cstar = nchunk - 1;
-    while (cstar > 0 && !(rec[cstar].s * expf(rec[cstar].m - M) > 0.f)) --cstar;
-    s_chunk = cstar;
-    s_before = 0;
-    s_redi[1] = 1;
+    s_chunk[warp] = cross ? cstar : -1;
+    s_before[warp] = before;
   }
   __syncthreads();
+  const unsigned found_w = __ballot_sync(0xffffffffu, lane < NW && s_chunk[lane % NW] >= 0);
+  const bool fallback = found_w == 0;
+  int cstar = fallback ? -1 : s_chunk[__ffs(found_w) - 1];
+  const Acc before = fallback ? (Acc)0 : s_before[__ffs(found_w) - 1];
+  if (fallback) {
+    // no crossing at all (z near 1): the last chunk with mass, last id in it
+    cstar = nchunk - 1;
+    while (cstar > 0 && !(rec[cstar].s * expf(rec[cstar].m - M) > 0.f)) --cstar;
+  }
 
   // 3) recompute chunk c*'s 32 logits (each warp 4 ids, lanes along d with
   //    16-byte loads), then warp 0 locates the token in id order
   __shared__ float s_logit[kChunk];
-  const int cstar = s_chunk;
   {
     // the warp's NQ ids side by side, so their weight loads are in flight together
     const TA* hr = head_in + (size_t)hrow * d;
@@ -612,8 +640,7 @@ k_head_select(const HeadRec* __restrict__ rec_all, int nchunk, const TA* __restr
     Acc y = __shfl_up_sync(0xffffffffu, pre, o);
     if (lane >= o) pre += y;
   }
-  const Acc Tp = s_T - s_before;
-  const bool fallback = s_redi[1] != 0;
+  const Acc Tp = T - before;
   unsigned hit = __ballot_sync(0xffffffffu, !fallback && (v < V) && (pre > Tp));
   unsigned pos = __ballot_sync(0xffffffffu, (v < V) && (e > (Acc)0));
   if (lane == 0) {
@@ -630,17 +657,22 @@ void launch_head_select(bool bf16, int n_rows, const HeadRec* rec, int nchunk, c
                         const float* noise, int32_t* tokens, int mtp_rows, size_t head_stride,
                         const int* err, const StepCommit& cm, cudaStream_t s) {
   if (n_rows == 0) return;
-  auto bf = [&](auto kern, int nt) {
-    kf_launch(kern, dim3(n_rows), dim3(nt), 0, s, rec, nchunk, (const __nv_bfloat16*)head_in, d,
-              (const __nv_bfloat16*)w_head, V, inv_tau, map_kind, noise, tokens, mtp_rows, head_stride, err, cm);
+  const int bytes = nchunk * (int)sizeof(HeadRec);
+  auto go = [&](auto kern, int nt, auto* in, auto* w) {
+    const int staged = bytes <= kSelStageMax && ceil_div(nchunk, nt) <= kSelKeep;
+    kf_launch(kern, dim3(n_rows), dim3(nt), staged ? bytes : 0, s, rec, nchunk, in, d, w, V, inv_tau, map_kind,
+              noise, tokens, mtp_rows, head_stride, err, cm, staged);
   };
-  if (bf16 && n_rows <= kSelWideRows)
-    bf(k_head_select<__nv_bfloat16, 2 * kSelThreads>, 2 * kSelThreads);
-  else if (bf16)
-    bf(k_head_select<__nv_bfloat16, kSelThreads>, kSelThreads);
-  else
-    kf_launch(k_head_select<float, kSelThreads>, dim3(n_rows), dim3(kSelThreads), 0, s, rec, nchunk, (const float*)head_in, d,
-        (const float*)w_head, V, inv_tau, map_kind, noise, tokens, mtp_rows, head_stride, err, cm);
+  if (bf16) {
+    auto* in = (const __nv_bfloat16*)head_in;
+    auto* w = (const __nv_bfloat16*)w_head;
+    if (n_rows <= kSelWideRows)
+      go(k_head_select<__nv_bfloat16, 2 * kSelThreads>, 2 * kSelThreads, in, w);
+    else
+      go(k_head_select<__nv_bfloat16, kSelThreads>, kSelThreads, in, w);
+  } else {
+    go(k_head_select<float, kSelThreads>, kSelThreads, (const float*)head_in, (const float*)w_head);
+  }
 }
 
 }  // namespace kf

@@ -48,6 +48,18 @@ def test_head_records_at_edges(head_env, rows, V, d, map_kind):  # noqa: F811
     assert check_against_oracle(x, w, z, 1.0, map_kind, got) == 0
 
 
+# the selection's record paths: 256 threads per row with 2048 chunks (8 records a
+# thread, staged) and 2049 (read in place); 512 threads with 2560 chunks (40 KB, the
+# most staged), 2561 (in registers, not staged) and 4097 (read in place)
+@pytest.mark.parametrize("rows,V", [(513, 65536), (513, 65540), (5, 81920), (5, 81921), (3, 131073)])
+@pytest.mark.parametrize("map_kind", [0, 1])
+def test_selection_record_paths(head_env, rows, V, map_kind):  # noqa: F811
+    torch, lib = head_env
+    x, w, z = _case(torch, rows, V, 64, rows + V)
+    got = run_op(lib, torch, x, w, z, 1.0, map_kind)
+    assert check_against_oracle(x, w, z, 1.0, map_kind, got) == 0
+
+
 @pytest.mark.parametrize("ids", [(5, 9), (31, 32), (40, 95), (64, 998)])
 def test_argmax_ties_take_the_lowest_id(head_env, ids):  # noqa: F811
     torch, lib = head_env
