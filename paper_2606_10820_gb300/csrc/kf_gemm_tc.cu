@@ -1386,9 +1386,7 @@ int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   // More than a wave of 256-wide tiles: a persistent loop whose epilogues
   // overlap the next tile's mainloop (OWT-shaped batch 512, k = 4: QKV 35.1 ->
   // 30.1 us, MLP-up 38.2 -> 30.7 us per layer).  Within one wave a CTA per
-  // tile keeps a fourth pipeline stage and has nothing to overlap.  The
-  // LM-head records keep their kernel, which streams each weight tile once
-  // per 256 rows.
+  // tile keeps a fourth pipeline stage and has nothing to overlap.
   // One wave of 256-wide tiles that leaves SMs idle, where 192-wide tiles
   // still fit one wave: the narrower tiles (the OWT-shaped O projection and
   // MLP-down at 4096 rows: 128 CTAs of 128 x 192 instead of 96 of 128 x 256;
