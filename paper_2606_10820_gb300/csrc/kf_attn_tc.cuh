@@ -463,7 +463,9 @@ k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args 
         tmem_ld32(lane_base + kColO + 32, o + 32);
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         arrive(o_free);
-        if (v.ctx >= 0 && l > 0.f) P::store(a, im, row, o, 1.f / l);
+        // every row of the item is written: one whose scores are NaN as NaN, not left
+        // as the buffer was (a row with finite scores has l > 0)
+        if (v.ctx >= 0) P::store(a, im, row, o, 1.f / l);
       }
     }
   }

@@ -73,3 +73,30 @@ def test_reference_maximum_moves(env, scale, step):  # noqa: F811
     ref = _reference(torch, *(x.float().cpu().numpy() for x in (q, kk, v)), ta.mask_full(N, k, 1))
     assert torch.isfinite(out).all()
     assert np.abs(out.cpu().numpy() - ref).max() <= 8e-3 * v.float().abs().max().item()
+
+
+def _attend(torch, lib, q, kk, v, N, k):
+    B, T, H, _ = q.shape
+    out = torch.full((B, T, H, 64), 7.0, device="cuda")
+    assert lib.kf_op_train_attention(1, B, H, N, k, 0, T, q.data_ptr(), kk.data_ptr(), v.data_ptr(),
+                                     out.data_ptr(), 0, None) == 0
+    torch.cuda.synchronize()
+    return out
+
+
+def test_nan_rows_are_written(env):  # noqa: F811
+    """A row whose scores are NaN comes out as NaN, not as what the caller's
+    buffer held, and no other row changes."""
+    torch, lib = env
+    N, k = 150, 3
+    T = N * (1 + k)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q, kk, v = (torch.randn(1, T, 2, 64, device="cuda", generator=g).to(torch.bfloat16) for _ in range(3))
+    want = _attend(torch, lib, q, kk, v, N, k)
+    rows = torch.tensor([3, 140, N + 1, T - 1], device="cuda")
+    q[0, rows, 1, 0] = float("nan")
+    out = _attend(torch, lib, q, kk, v, N, k)
+    assert torch.isnan(out[0, rows, 1]).all()
+    want[0, rows, 1] = 0
+    out[0, rows, 1] = 0
+    assert torch.equal(out, want)
