@@ -26,7 +26,7 @@ struct PrefillPolicy {
   struct Maps { CUtensorMap kv; };     // this layer's pages as rows of 64 bf16
   struct Item { int slot, row0, rows, pos0, h; };
   struct TileRef { int page; uint32_t mask; };   // this lane's page, the lanes that copy one
-  static constexpr bool kQByRows = true, kZeroV = true, kWindows = false;
+  static constexpr bool kQByRows = true, kWindows = false;
 
   static __device__ __forceinline__ int n_items(const Args& a) { return a.n_groups * a.H; }
   static __device__ __forceinline__ bool all_open(const Args&) { return true; }
@@ -79,6 +79,19 @@ struct PrefillPolicy {
   static __device__ __forceinline__ void load_v(const Maps& m, const Args& a, const Item& im, const TileRef& r, int lane,
                                                 uint32_t dst, uint32_t bar) {
     if (r.page >= 0) tma_load_2d(dst + lane * kPageBytes, &m.kv, bar, 0, ((r.page * 2 + 1) * a.H + im.h) * kPage);
+  }
+  // The pages that are not copied (past the last key) are cleared for each tile:
+  // their probabilities are 0 and 0 * V must be 0, and the stage may hold another
+  // sequence's values, which need not be finite
+  static __device__ __forceinline__ void clear_v(const TileRef& r, int lane, uint8_t* dst) {
+    if (r.mask == (1u << (fa::kKeys / kPage)) - 1) return;
+    for (int p = 0; p < fa::kKeys / kPage; ++p)
+      if (!((r.mask >> p) & 1u))
+#pragma unroll
+        for (int i = 0; i < (int)kPageBytes; i += 32 * 16)
+          *reinterpret_cast<uint4*>(dst + p * kPageBytes + i + 16 * lane) = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
   }
   static __device__ __forceinline__ void store(const Args& a, const Item& im, int row, const float* o, float inv) {
     uint4* dst = reinterpret_cast<uint4*>(a.out + ((size_t)(im.row0 + row) * a.H + im.h) * fa::kHD);

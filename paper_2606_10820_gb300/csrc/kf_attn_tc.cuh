@@ -108,7 +108,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //   n_items(a)
 //   kQByRows             false: load_q(maps, it, sQ, bar) by lane 0 of warp 0 (kTileBytes);
 //                        true: q_rows(a, it, sm, first, lane): 32 rows by each softmax warp
-//   kv_bytes / load_kv   the bytes of a K (or V) tile and its copies, by warp 0's lanes
+//   tile(a, it, kt, kend, lane, d_err)   what a key tile copies: TileRef, by warp 0's lanes
+//   tile_bytes / load_k / load_v   the bytes of a K (or V) tile and its copies
+//   clear_v(ref, lane, dst)   the V rows that no copy of this tile writes become zeros
 //   vis(a, it, row)      the row's visible keys (ctx = -1: no such row)
 //   store(a, it, row, o, inv)   the finished row
 template <class P>
@@ -165,13 +167,6 @@ k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args 
     mbar_init(smem_u32(o_free), kSoftWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (P::kZeroV) {
-    // V rows that no copy writes (past the last key) stay finite: their
-    // probabilities are 0 and 0 * V must be 0
-    for (int i = t; i < (int)(kVSt * kTileBytes / 16); i += kThreads)
-      reinterpret_cast<uint4*>(sm + (1 + kKSt) * kTileBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(kTmemCols)
@@ -213,6 +208,7 @@ k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args 
         k_issued = g + 1;
         ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&v_empty[vs]), ((g / kVSt) & 1) ^ 1, d_err));
         if (!ok) break;
+        P::clear_v(ref, lane, sm + (1 + kKSt + vs) * kTileBytes);
         if (lane == 0) mbar_expect_tx(smem_u32(&v_full[vs]), P::tile_bytes(ref));
         __syncwarp();
         P::load_v(maps, a, im, ref, lane, sV + vs * kTileBytes, smem_u32(&v_full[vs]));

@@ -308,7 +308,7 @@ struct TrainPolicy {
   struct Maps { CUtensorMap q, k, v; };
   struct Item { int q0, q1, h, b; };     // rows q0 .. q1 - 1 (at most 128)
   struct TileRef { int kt; };
-  static constexpr bool kQByRows = false, kZeroV = false, kWindows = true;
+  static constexpr bool kQByRows = false, kWindows = true;
 
   static __device__ __forceinline__ int n_items(const Args& g) { return g.n_qt * g.a.H * g.n_batch; }
   static __device__ __forceinline__ bool all_open(const Args& g) { return !g.a.dense; }
@@ -377,6 +377,7 @@ struct TrainPolicy {
                                                 uint32_t dst, uint32_t bar) {
     if (lane == 0) tma_load_4d(dst, &m.v, bar, 0, im.h, r.kt, im.b);
   }
+  static __device__ __forceinline__ void clear_v(const TileRef&, int, uint8_t*) {}   // (a copy fills the tile)
   static __device__ __forceinline__ void store(const Args& g, const Item& im, int row, const float* o, float inv) {
     const TrainAttnArgs& a = g.a;
     float* dst = a.out + (((size_t)im.b * (a.q_end - a.q_begin) + (im.q0 + row - a.q_begin)) * a.H + im.h) * kHD;

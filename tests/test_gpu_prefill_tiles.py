@@ -47,3 +47,27 @@ def test_prefill_items(kf, lens, prefill_rows):
     _, rl = ref.step(0, z, want_logits=True)
     assert logit_check(lg, rl) <= LOGIT_TOL
     dec.close()
+
+
+def test_nan_sequence_stays_alone(kf):
+    """A prompt whose keys and values are NaN leaves the other prompts of the
+    batch unchanged: 1,200 later items of 100 keys reuse the value tiles of 312
+    items of 128 keys whose last row is NaN (the last token of a prompt is not
+    prefilled: it is the first step's)."""
+    w = make_weights(CFG)
+    w["tok_emb"] = w["tok_emb"].copy()
+    w["tok_emb"][7] = np.nan
+    bad, good = 26, 100
+    prompts = [np.where(p == 7, 8, p) for p in make_prompts([129] * bad + [101] * good, CFG.vocab)]
+    z = np.random.default_rng(1).random((bad + good, 1), dtype=np.float32)
+    got = []
+    for last in (8, 7):
+        for p in prompts[:bad]:
+            p[-2] = last
+        dec = kf.Decoder(CFG, w, max_batch=bad + good, max_k=2, prefill_rows=16384)
+        dec.prefill(prompts)
+        dec.step(0, z)
+        got.append(np.array(dec.logits(1))[bad:])
+        dec.close()
+    assert np.isfinite(got[0]).all()
+    assert np.array_equal(got[0], got[1])
