@@ -100,3 +100,21 @@ def test_nan_rows_are_written(env):  # noqa: F811
     want[0, rows, 1] = 0
     out[0, rows, 1] = 0
     assert torch.equal(out, want)
+
+
+def test_large_values_stay_finite(env):  # noqa: F811
+    """Scores that rise by 2^60 along the context with V near 2^100: probabilities
+    taken against the first tile's maximum would overflow the sum of P V."""
+    torch, lib = env
+    N, k = 520, 2
+    T = N * (1 + k)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, kk, v = (torch.randn(1, T, 1, 64, device="cuda", generator=g) for _ in range(3))
+    q[..., 0] = 8.0
+    kk *= 0.1
+    kk[0, :, 0, 0] = 165.0 / T * torch.arange(T, device="cuda")
+    q, kk, v = (x.to(torch.bfloat16) for x in (q, kk, v * 2.0 ** 100))
+    out = _attend(torch, lib, q, kk, v, N, k)
+    ref = _reference(torch, *(x.float().cpu().numpy() for x in (q, kk, v)), ta.mask_full(N, k, 1))
+    assert torch.isfinite(out).all()
+    assert np.abs(out.cpu().numpy() - ref).max() <= 8e-3 * v.float().abs().max().item()
