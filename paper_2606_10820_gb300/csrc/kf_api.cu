@@ -18,7 +18,6 @@ using namespace kf;
 
 namespace kf {
 thread_local bool g_pdl = false;
-thread_local int g_gemm_flags = 0;
 }
 
 namespace kf {
@@ -203,9 +202,9 @@ static void gemm(kf_ctx* c, int kind, int M, int N, int K, const void* A, int ld
   GemmDesc g{M, N, K, A, lda, W, ldw, e};
   g.l2_next = l2_next;
   g.l2_bytes = l2_bytes;
+  g.per_tile = c->cfg.flags & KF_FLAG_NO_PERSISTENT_GEMM;
   prof_begin(c, kind);
   bool use_tc = c->bf16 && !(c->cfg.flags & KF_FLAG_SIMT_GEMM) && tc_gemm_supported(g);
-  g_gemm_flags = (c->cfg.flags & KF_FLAG_NO_PERSISTENT_GEMM) ? kGemmNoPersist : 0;
   if (c->skinny && e.kind != EPI_HEAD && e.kind != EPI_LOGITS) {
     // every projection of a skinny enqueue must take this path: the fused
     // RMSNorm's producers and consumers agree on it

@@ -1314,7 +1314,7 @@ int active_clusters(int cs) {
 
 int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   const int num_sms = device_sms();
-  const bool persist = !(g_gemm_flags & kGemmNoPersist);
+  const bool persist = !g.per_tile;
   // CTA pairs past a wave of one-CTA tiles (those never split K), where their
   // rounds of 256 x 256 tiles are many and deep enough to outweigh the pair's
   // start (about 4 us) and its coarser rounds.  One-CTA loop -> pairs,
@@ -1396,7 +1396,7 @@ int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   if (ceil_div(g.N, 256) * m_tiles <= num_sms && ceil_div(g.N, 192) * m_tiles <= num_sms &&
       ceil_div(g.N, 192) > ceil_div(g.N, 256))
     return launch_bn<192, 5, 1>(g, d_err, num_sms, s);
-  if (g.epi.kind != EPI_HEAD && !(g_gemm_flags & kGemmNoPersist) && ceil_div(g.N, 256) * m_tiles > num_sms)
+  if (g.epi.kind != EPI_HEAD && persist && ceil_div(g.N, 256) * m_tiles > num_sms)
     return launch_persist<256, 3>(g, d_err, num_sms, s);
   return launch_bn<256, 4, 1>(g, d_err, num_sms, s);
 }

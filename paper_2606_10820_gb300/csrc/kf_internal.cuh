@@ -410,9 +410,6 @@ struct PdlScope {
   explicit PdlScope(bool on) : prev(g_pdl) { g_pdl = on; }
   ~PdlScope() { g_pdl = prev; }
 };
-// tensor-core GEMM launch options for the launches made by this thread
-constexpr int kGemmNoPersist = 1;  // one CTA per tile even past a wave of tiles
-extern thread_local int g_gemm_flags;
 
 template <typename... KArgs, typename... Args>
 inline void kf_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -445,6 +442,8 @@ struct GemmDesc {
   // points: a clearing memset of its own before each call cost about 2 us).
   // Its kernels set the word only after a wait of about 2 s
   bool clear_err = false;
+  // tensor-core GEMM: one CTA per tile even past a wave of tiles
+  bool per_tile = false;
 };
 
 // SIMT GEMM (bf16 operands; fp32 accumulation, k ascending per output)

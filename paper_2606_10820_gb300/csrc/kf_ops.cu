@@ -97,7 +97,7 @@ extern "C" int kf_op_gemm_bf16(int32_t impl, int32_t M, int32_t N, int32_t K, co
   cudaStream_t s = (cudaStream_t)stream;
   if (impl == KF_GEMM_TCGEN05 || impl == KF_GEMM_TCGEN05_PER_TILE) {
     if (!tc_gemm_supported(g)) return KF_E_ARG;
-    g_gemm_flags = impl == KF_GEMM_TCGEN05_PER_TILE ? kGemmNoPersist : 0;
+    g.per_tile = impl == KF_GEMM_TCGEN05_PER_TILE;
     int* err = op_error_word(s, false);
     if (!err) return KF_E_CUDA;
     g.clear_err = true;
