@@ -27,10 +27,11 @@ extern "C" {
  * A, W: bf16, row-major, rows 16-byte aligned; K a multiple of 64 for
  * KF_GEMM_TCGEN05 and KF_GEMM_SKINNY (which also needs M <= 64), N a
  * multiple of 4.  out: fp32 row-major [M][N].  The first
- * call on a device allocates a 4-byte device error word for that device that
- * lives until process exit; each call clears it on `stream` (the tcgen05
- * kernels as they start), and the kernel ORs its error bits into it (a
- * bounded pipeline wait that ran out).  Asynchronous: kf_op_status(stream) reports
+ * tcgen05 or skinny call on a device allocates a 4-byte device error word for
+ * that device that lives until process exit; each such call clears it on
+ * `stream` (the tcgen05 kernels as they start) and ORs its error bits into it
+ * (a bounded pipeline wait that ran out).  KF_GEMM_SIMT, and a call refused
+ * with KF_E_ARG, leave it alone.  Asynchronous: kf_op_status(stream) reports
  * those errors.  Errors: KF_E_ARG (shapes / alignment), KF_E_CUDA.
  */
 int kf_op_gemm_bf16(int32_t impl, int32_t M, int32_t N, int32_t K, const void* A, const void* W,

@@ -59,6 +59,14 @@ int* op_error_word(cudaStream_t s, bool clear) {
 }
 }  // namespace kf
 
+// `code` for a call whose first kernel, which clears the error word, did not
+// start: the word is cleared here, so that kf_op_status does not report an
+// earlier call's errors for this one
+static int not_run(int* err, cudaStream_t s, int code) {
+  cudaMemsetAsync(err, 0, sizeof(int), s);
+  return code;
+}
+
 // the LM-head GEMM with the chunk-record epilogue, then the token select
 static int head_tokens(int32_t rows, int32_t V, int32_t d, const void* x, const void* w_head,
                        const float* noise, float tau, int32_t map_kind, int32_t* tokens,
@@ -72,8 +80,8 @@ static int head_tokens(int32_t rows, int32_t V, int32_t d, const void* x, const 
   g.epi.nchunk = nchunk;
   g.epi.want_arg = map_kind == KF_MAP_ARGMAX;
   g.clear_err = true;
-  if (!tc_gemm_supported(g)) return KF_E_ARG;
-  if (launch_gemm_tc(g, err, s) != 0) return KF_E_CUDA;
+  if (!tc_gemm_supported(g)) return not_run(err, s, KF_E_ARG);
+  if (launch_gemm_tc(g, err, s) != 0) return not_run(err, s, KF_E_CUDA);
   // the token selection waits for the records itself: its launch overlaps them
   const PdlScope pdl(true);
   launch_head_select(true, rows, rec, nchunk, x, d, w_head, V, 1.0f / tau, map_kind, noise, tokens, 0, 0,
@@ -101,7 +109,7 @@ extern "C" int kf_op_gemm_bf16(int32_t impl, int32_t M, int32_t N, int32_t K, co
     int* err = op_error_word(s, false);
     if (!err) return KF_E_CUDA;
     g.clear_err = true;
-    if (launch_gemm_tc(g, err, s) != 0) return KF_E_CUDA;
+    if (launch_gemm_tc(g, err, s) != 0) return not_run(err, s, KF_E_CUDA);
   } else if (impl == KF_GEMM_SKINNY) {
     if (!skinny_gemm_supported(g)) return KF_E_ARG;
     int* err = op_error_word(s);

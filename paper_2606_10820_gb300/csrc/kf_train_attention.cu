@@ -450,13 +450,16 @@ extern "C" int kf_op_train_attention(int32_t blocks, int32_t B, int32_t H, int32
     for (int i = 0; i < g.n_qt; ++i) g.q0[i] = tiles[i].second;
   }
   const long long items = (long long)g.n_qt * H * B;
-  if (items > (1ll << 30)) return KF_E_ARG;
-  int* err = op_error_word(s, false);   // cleared by the kernel
+  const bool fits = items <= (1ll << 30);
+  int* err = op_error_word(s, !fits);   // cleared by the kernel, if it runs
   if (!err) return KF_E_CUDA;
+  if (!fits) return KF_E_ARG;
   static PerDevice attr_tc;
   set_smem_attr(attr_tc, fa::k_attn_tc<TrainPolicy>, fa::kSmemBytes);
   // persistent: two CTAs per SM over the (query tile, head, sequence) items
   const dim3 grid((unsigned)std::min<long long>(items, 2ll * device_sms()));
   kf_launch(fa::k_attn_tc<TrainPolicy>, grid, dim3(fa::kThreads), fa::kSmemBytes, s, maps, g, err, 1);
-  return cudaGetLastError() == cudaSuccess ? KF_OK : KF_E_CUDA;
+  if (cudaGetLastError() == cudaSuccess) return KF_OK;
+  op_error_word(s);
+  return KF_E_CUDA;
 }

@@ -1,10 +1,13 @@
 """Host code of the entry points, without a GPU (host_calls.py)."""
+import ctypes
+
 import pytest
 
 import host_calls
 from host_calls import launches
 
 GEMM_TC, GEMM_PER_TILE = 0, 2
+KF_E_ARG, KF_E_CUDA = -1, -4
 P = 4096        # a 16-byte aligned device address that nothing reads
 
 
@@ -29,3 +32,28 @@ def test_head_after_a_per_tile_product(lib, fn):
     assert "k_gemm_tc<" in launches(lib)[0].kernel
     assert _head(lib, *shape, fn=fn) == 0
     assert launches(lib) == want
+
+
+def test_refused_calls_leave_no_earlier_error(lib):
+    """An op that is refused, or whose launch fails, has cleared the error word
+    of the calls before it: kf_op_status reports this call's errors only."""
+    assert _head(lib, 8, 1000, 768) == 0           # (allocates the word)
+    word = ctypes.cast(lib.fake_last_alloc(4), ctypes.POINTER(ctypes.c_int))
+
+    def train(heads):
+        return lib.kf_op_train_attention(1, 1 << 15, heads, 64, 4, 0, 320, P, P, P, P, 0, None)
+
+    def fails(call):
+        lib.fake_launches_left(0)
+        try:
+            return call()
+        finally:
+            lib.fake_launches_left(-1)
+
+    for call, code in ((lambda: _head(lib, 8, 1000, 768, x=P + 2), KF_E_ARG),        # misaligned rows
+                       (lambda: train(1 << 15), KF_E_ARG),                           # too many items
+                       (lambda: fails(lambda: _head(lib, 8, 1000, 768)), KF_E_CUDA),
+                       (lambda: fails(lambda: lib.kf_op_gemm_bf16(GEMM_TC, 64, 64, 64, P, P, P, None)), KF_E_CUDA)):
+        word[0] = 1
+        assert call() == code
+        assert lib.kf_op_status(None) == 0
