@@ -1325,13 +1325,17 @@ int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   // Records and logits: 2048 x 50,257 at K = 1024 162 -> 146, K = 768 147 -> 134,
   // 1024 x 50,257 x 768 (11 rounds) 74.3 -> 71.5, 512 x 50,257 x 1024 (6) 57.3 ->
   // 52.7; but 1024 x 30,522 x 768 (7) 47.6 -> 51.5, 2100 x 50,257 x 256 82 -> 99;
-  // logits 2048 x 50,257 197 -> 179.
+  // logits 2048 x 50,257 197 -> 179.  Not with one or three row tiles, where half or a
+  // quarter of the pairs' CTAs have no rows (LM head and selection, greedy: 1 row x
+  // 50,257 x 2048 48 -> 64, 1 x 131,072 x 1024 56 -> 80, 300 x 131,072 x 512 57 -> 68,
+  // 300 x 50,257 x 1024 38 -> 44).
   if (persist && ceil_div(g.N, 256) * ceil_div(g.M, kBM) > num_sms && num_sms >= 2) {
     const int rounds = ceil_div(ceil_div(g.N, 256) * ceil_div(g.M, 2 * kBM), num_sms / 2);
     const long long depth = (long long)rounds * g.K;
     const bool deep = depth >= 6144 || (g.K >= 1024 && depth >= 4096);
-    if (g.epi.kind == EPI_HEAD && deep) return launch_pair_epi<256, 6, EPI_HEAD>(g, d_err, num_sms, s);
-    if (g.epi.kind == EPI_LOGITS && deep) return launch_pair_epi<256, 4, EPI_LOGITS>(g, d_err, num_sms, s);
+    const bool filled = 5 * ceil_div(g.M, kBM) >= 8 * ceil_div(g.M, 2 * kBM);
+    if (g.epi.kind == EPI_HEAD && deep && filled) return launch_pair_epi<256, 6, EPI_HEAD>(g, d_err, num_sms, s);
+    if (g.epi.kind == EPI_LOGITS && deep && filled) return launch_pair_epi<256, 4, EPI_LOGITS>(g, d_err, num_sms, s);
     if (pair_rows_ok(g) && g.K >= 768 && (rounds >= 3 || deep)) {
       if (g.epi.kind == EPI_STORE_F32) return launch_pair_epi<256, 6, EPI_STORE_F32>(g, d_err, num_sms, s);
       if (g.epi.kind == EPI_BIAS_GELU) return launch_pair_epi<256, 6, EPI_BIAS_GELU>(g, d_err, num_sms, s);

@@ -16,6 +16,11 @@ def lib(tmp_path_factory):
     return host_calls.load(str(tmp_path_factory.mktemp("host")))
 
 
+@pytest.fixture(autouse=True)
+def _fresh(lib):
+    lib.fake_clear()
+
+
 def _head(lib, rows, V, d, map_kind=0, x=P, fn="kf_op_head_tokens"):
     return getattr(lib, fn)(rows, V, d, x, P, P, 1.0, map_kind, P, None)
 
@@ -57,3 +62,16 @@ def test_refused_calls_leave_no_earlier_error(lib):
         word[0] = 1
         assert call() == code
         assert lib.kf_op_status(None) == 0
+
+
+@pytest.mark.parametrize("rows,V,d,kernel", [
+    (1, 50257, 2048, "persist<128"), (128, 131072, 1024, "persist<128"),     # one row tile
+    (257, 131072, 512, "persist<256"), (384, 50257, 1024, "persist<256"),    # three: the last pair's second CTA is empty
+    (129, 131072, 1024, "pair<"), (256, 131072, 1024, "pair<"), (385, 50257, 1024, "pair<"),
+    (513, 50257, 1024, "pair<"),                                             # five
+])
+def test_heads_stay_off_pairs_without_rows(lib, rows, V, d, kernel):
+    """Heads of one or three row tiles leave CTAs of a pair without rows: they run
+    on the one-CTA loops."""
+    assert _head(lib, rows, V, d) == 0
+    assert kernel in launches(lib)[0].kernel
