@@ -442,13 +442,15 @@ template <int EPI>
 static int launch_skinny_epi(const GemmDesc& g, int* d_err, cudaStream_t s) {
   int splits, kc, m_pad;
   skinny_plan(g, &splits, &kc, &m_pad);
-  // At most three CTAs per SM.  Launched dependently, while the kernel before
+  // Launched dependently, at most three CTAs per SM: while the kernel before
   // holds one CTA on most SMs, smaller CTAs piled up on the few SMs that it left
-  // free (five or six each) and the kernel ended with those: padding from 36 KB
-  // took two calls of one sequence at k = 4 from 625 to 595 us, of two sequences
-  // 751 -> 714, the AR step of 16 785 -> 748; 50 KB helps one sequence only, 112 KB
-  // delays the CTAs past the first of an SM (the AR step of 16: 768)
-  const size_t smem = std::max(skinny_smem(kc, m_pad), (size_t)74 * 1024);
+  // free (five or six each) and the kernel ended with those.  Two calls of the
+  // 768-wide 12-layer model, unpadded -> padded: four sequences at k = 1 654 -> 612
+  // us, the AR step of 16 784 -> 751, one and eight at k = 4 the same (595, 853).
+  // 112 KB delays the CTAs past the first of an SM (the AR step of 16: 768).  By
+  // itself a product has the SMs free and the limit only costs (32 x 1024 x 3072
+  // 10.4 us, padded 13.8; 5 x 50,304 x 256 17.9, padded 22.4).
+  const size_t smem = std::max(skinny_smem(kc, m_pad), g_pdl ? (size_t)74 * 1024 : 0);
   if (smem > 200 * 1024) return -1;
   static PerDevice attr;
   set_smem_attr(attr, k_gemm_skinny<EPI>, smem);

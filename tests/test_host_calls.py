@@ -6,7 +6,7 @@ import pytest
 import host_calls
 from host_calls import launches
 
-GEMM_TC, GEMM_PER_TILE = 0, 2
+GEMM_TC, GEMM_PER_TILE, GEMM_SKINNY = 0, 2, 3
 KF_E_ARG, KF_E_CUDA = -1, -4
 P = 4096        # a 16-byte aligned device address that nothing reads
 
@@ -75,3 +75,13 @@ def test_heads_stay_off_pairs_without_rows(lib, rows, V, d, kernel):
     on the one-CTA loops."""
     assert _head(lib, rows, V, d) == 0
     assert kernel in launches(lib)[0].kernel
+
+
+@pytest.mark.parametrize("M,N,K", [(32, 1024, 3072), (5, 50304, 256), (1, 2304, 768), (64, 64, 64)])
+def test_skinny_product_is_not_padded(lib, M, N, K):
+    """Shared memory that keeps a dependent launch's CTAs apart is not asked for
+    by a product that runs by itself: its A and W rows of the split and 12 KB."""
+    assert lib.kf_op_gemm_bf16(GEMM_SKINNY, M, N, K, P, P, P, None) == 0
+    (got,) = launches(lib)
+    assert "skinny" in got.kernel
+    assert got.smem <= K // got.cluster * 2 * (16 + (M + 7) // 8 * 8) + 12 * 1024
