@@ -78,8 +78,9 @@ typedef struct kf_config {
   int32_t page_size;    /* tokens per KV page; must be 16                     */
   int32_t n_pages;      /* KV pool size in pages; 0 => enough for max_batch
                            sequences of max_len tokens                        */
-  int32_t prefill_rows; /* rows per prefill chunk; 0 => 4096 (a remainder of up
-                           to a quarter of a chunk joins the last one)        */
+  int32_t prefill_rows; /* most rows of a prefill chunk, in multiples of 128;
+                           0 => 4096, and a remainder of up to 1024 rows
+                           joins the last chunk                               */
   int32_t flags;        /* KF_FLAG_*                                          */
   float tau;            /* temperature: logits are divided by tau (> 0)       */
   float rms_eps;        /* RMSNorm epsilon                                    */

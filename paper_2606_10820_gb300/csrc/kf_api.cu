@@ -82,6 +82,7 @@ struct kf_ctx {
   int pend_stride = 8;
   // workspaces
   int R_cap = 0, NR_cap = 0, prefill_rows = 0;
+  int last_chunk_rows = 0;      // the most rows of a prefill's last chunk
   bool fused = false;     // RMSNorm fused into the tcgen05 GEMMs (bf16, head_dim 64)
   // The projections of the layers being enqueued run as skinny warp-MMA
   // kernels (at most 64 rows, fused path): their norm consumers take the
@@ -467,13 +468,6 @@ static int upload_page_row(kf_ctx* c, int b) {
   return KF_OK;
 }
 
-// The most rows of a prefill's last chunk: a remainder of up to a quarter of a
-// chunk joins it, because a chunk of few rows is a chain of five launches per
-// layer that leaves the chip idle (768-wide, 12 layers, microseconds per prefill
-// with the remainder apart -> joined: 5 prompts of 1000 2380 -> 1821, 16 of 539
-// 3289 -> 2889).
-static int last_chunk_rows(const kf_ctx* c) { return c->prefill_rows + c->prefill_rows / 4; }
-
 // ------------------------------------------------------------- C ABI
 extern "C" {
 
@@ -668,7 +662,13 @@ int kf_init(const kf_config* cfg_in, const kf_weights* w, void* stream, kf_ctx**
   c->pend_stride = MK;
   c->NR_cap = round_up(MB * MK, 128);
   c->prefill_rows = round_up(cfg.prefill_rows, 128);
-  c->R_cap = std::max(round_up(MB * 2 * MK, 128), round_up(last_chunk_rows(c), 128));
+  // By default a remainder of up to a quarter of a chunk joins the last chunk,
+  // because a chunk of few rows is a chain of five launches per layer that leaves
+  // the chip idle (768-wide, 12 layers, microseconds per prefill with the remainder
+  // apart -> joined: 5 prompts of 1000 2380 -> 1821, 16 of 539 3289 -> 2889).  A
+  // caller's prefill_rows bounds every chunk, and with it the row workspaces.
+  c->last_chunk_rows = c->prefill_rows + (cfg_in->prefill_rows == 0 ? c->prefill_rows / 4 : 0);
+  c->R_cap = std::max(round_up(MB * 2 * MK, 128), c->last_chunk_rows);
   const int R = c->R_cap;
   if ((r = dalloc(c, &c->d_len, MB * 4)) || (r = dalloc(c, &c->d_len0, MB * 4)) ||
       (r = dalloc(c, &c->d_order, MB * 4)) ||
@@ -702,10 +702,6 @@ int kf_init(const kf_config* cfg_in, const kf_weights* w, void* stream, kf_ctx**
   return KF_OK;
 }
 
-// Prefill: the KV of each listed slot's first n tokens (positions 0..n-1),
-// in row chunks of prefill_rows (the last one up to last_chunk_rows), attention
-// groups of consecutive rows of a sequence: up to 128 for the tcgen05 kernel,
-// else up to 16.  The slots' pages must be allocated and uploaded.
 // The rows of a chunk's attention groups: 128 (tcgen05) once the 128-row items
 // cover the SMs and hold 40 rows or more on average, else 16 (warp-level MMA, which
 // also splits the keys of few long rows).  Measured, 768-wide model, 4 layers,
@@ -722,6 +718,11 @@ static int prefill_group_rows(const kf_ctx* c, const std::vector<int4>& runs) {
   }
   return tiles * c->H >= c->num_sms && rows >= 40 * tiles ? kMaxTileRows : kMaxGroupRows;
 }
+
+// Prefill: the KV of each listed slot's first n tokens (positions 0..n-1),
+// in row chunks of prefill_rows (the last one up to last_chunk_rows), attention
+// groups of consecutive rows of a sequence: up to 128 for the tcgen05 kernel,
+// else up to 16.  The slots' pages must be allocated and uploaded.
 struct PrefillSeq {
   int slot;
   const int32_t* tok;
@@ -760,7 +761,7 @@ static int prefill_rows(kf_ctx* c, const std::vector<PrefillSeq>& seqs) {
   };
   long long left = 0;              // rows not yet in a flushed chunk
   for (const PrefillSeq& q : seqs) left += q.n;
-  auto chunk_rows = [&] { return left <= last_chunk_rows(c) ? (int)left : c->prefill_rows; };
+  auto chunk_rows = [&] { return left <= c->last_chunk_rows ? (int)left : c->prefill_rows; };
   int cap = chunk_rows();
   for (const PrefillSeq& q : seqs) {
     int p = 0;

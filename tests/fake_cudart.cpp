@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <iterator>
 #include <map>
 #include <new>
 #include <string>
@@ -26,7 +27,6 @@ std::map<size_t, void*>& last_alloc() {
   static std::map<size_t, void*> m;
   return m;
 }
-size_t g_total = 0;
 int g_launches_left = -1;          // launches that still succeed; -1: all
 thread_local bool g_heap_fails = false;
 struct Call {
@@ -64,8 +64,8 @@ const char* fake_launches() { return log().c_str(); }
 void fake_clear() { log().clear(); }
 void fake_launches_left(int n) { g_launches_left = n; }
 void fake_heap_fails(int on) { g_heap_fails = on != 0; }
+// the last live device allocation of that size
 void* fake_last_alloc(size_t bytes) { return last_alloc().count(bytes) ? last_alloc()[bytes] : nullptr; }
-size_t fake_allocated() { return g_total; }
 
 // ------------------------------------------------------------ the runtime
 void** __cudaRegisterFatBinary(void*) {
@@ -134,7 +134,6 @@ cudaError_t cudaMalloc(void** p, size_t n) {
   *p = aligned_alloc(256, (n + 255) / 256 * 256);
   if (!*p) return cudaErrorMemoryAllocation;
   last_alloc()[n] = *p;
-  g_total += n;
   return cudaSuccess;
 }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
@@ -142,6 +141,8 @@ cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
   return *p ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 cudaError_t cudaFree(void* p) {
+  for (auto it = last_alloc().begin(); it != last_alloc().end();)
+    it = it->second == p ? last_alloc().erase(it) : std::next(it);
   free(p);
   return cudaSuccess;
 }

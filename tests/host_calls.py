@@ -24,11 +24,15 @@ def load(tmp_path):
                         "-I", os.path.join(cuda, "include"), "-o", out, os.path.join(HERE, "fake_cudart.cpp"), *objs,
                         "-lpthread"], capture_output=True, text=True)
     assert p.returncode == 0, p.stderr
-    lib = ctypes.CDLL(out)
+    from paper_2606_10820_gb300 import kforcing as kf
+    loaded, kf._lib = kf._lib, None
+    try:
+        lib = kf.load_library(out)
+    finally:
+        kf._lib = loaded
     lib.fake_launches.restype = ctypes.c_char_p
     lib.fake_last_alloc.restype = ctypes.c_void_p
     lib.fake_last_alloc.argtypes = [ctypes.c_size_t]
-    lib.fake_allocated.restype = ctypes.c_size_t
     I32, VP, F32 = ctypes.c_int32, ctypes.c_void_p, ctypes.c_float
     lib.kf_op_gemm_bf16.argtypes = [I32] * 4 + [VP] * 4
     lib.kf_op_head_tokens.argtypes = [I32] * 3 + [VP] * 3 + [F32, I32, VP, VP]

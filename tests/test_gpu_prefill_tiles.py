@@ -31,8 +31,9 @@ def kf():
     ([130, 2, 17, 65, 128, 129, 256, 257, 258, 90, 80, 70, 60], 4096),   # remainders of 1 .. 127 rows
     ([150, 140, 131, 97, 200, 260, 75, 85, 95, 105] * 2, 1536),   # a prompt cut across chunks
     ([1000, 980], 1408),                                          # up to eight key tiles; a second chunk of few items
-    ([321] * 6, 1536),                                            # 1920 rows: the remainder of a quarter joins the chunk
-    ([321] * 5 + [322], 1536),                                    # 1921 rows: a second chunk of 385
+    ([321] * 16, 0),                                              # 5120 rows: the remainder of a quarter joins the chunk
+    ([321] * 15 + [322], 0),                                      # 5121 rows: a second chunk of 1025
+    ([321] * 6, 1536),                                            # 1920 rows: a second chunk of 384
 ])
 def test_prefill_items(kf, lens, prefill_rows):
     w = make_weights(CFG)

@@ -85,3 +85,31 @@ def test_skinny_product_is_not_padded(lib, M, N, K):
     (got,) = launches(lib)
     assert "skinny" in got.kernel
     assert got.smem <= K // got.cluster * 2 * (16 + (M + 7) // 8 * 8) + 12 * 1024
+
+
+@pytest.mark.parametrize("asked,lens,chunks", [
+    (0, [321] * 16, [5120]),                     # the default joins a remainder of up to a quarter
+    (0, [321] * 15 + [322], [4096, 1025]),
+    (1536, [321] * 6, [1536, 384]),              # a caller's size is the most rows of every chunk
+    (1536, [1537], [1536]),
+    (4096, [1025] * 5, [4096, 1024]),
+    (100, [201], [128, 72]),                     # (in multiples of 128)
+])
+def test_prefill_chunks(lib, monkeypatch, asked, lens, chunks):
+    """The rows of each prefill chunk (one embedding block per row), and the row
+    workspaces of a context, which hold no more than the largest chunk."""
+    import numpy as np
+    from paper_2606_10820_gb300 import kforcing as kf
+    from synth import OWT, make_prompts, make_weights
+    monkeypatch.setattr(kf, "_lib", lib)
+    cfg = OWT.replace(n_layer=1, d_model=64, n_head=1, d_ff=64, vocab=67, noise_hidden=64, max_len=2048)
+    dec = kf.Decoder(cfg, make_weights(cfg), max_batch=16, max_k=1, prefill_rows=asked)
+    cap = -(-(asked or 4096) // 128) * 128
+    rows = cap if asked else 5120
+    streams = [n for n in range(128, 6145, 128) if lib.fake_last_alloc(n * cfg.d_model * 4)]   # [rows][d] floats
+    assert rows in streams and -(-rows * 5 // 512) * 128 not in streams
+    lib.fake_clear()
+    dec.prefill(make_prompts(lens, cfg.vocab))
+    got = [x.grid[0] for x in launches(lib) if "embed_tokens" in x.kernel]
+    dec.close()
+    assert got == chunks
