@@ -27,8 +27,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <utility>
-#include <vector>
 
 #include "../../include/kforcing_ops.h"
 #include "kf_attn_tc.cuh"
@@ -439,15 +437,19 @@ extern "C" int kf_op_train_attention(int32_t blocks, int32_t B, int32_t H, int32
   }
   if (g.n_qt <= kTileList) {
     // sorted by the context keys a tile's last row sees (the windows add about
-    // the same to every block tile)
-    std::vector<std::pair<long long, int>> tiles;
+    // the same to every block tile), then by position; on the stack: nothing
+    // that throws lies between the C caller and the launch
+    struct Tile { long long keys; int q0; };
+    Tile tiles[kTileList];
+    int n = 0;
     for (int p = 0; p <= blocks; ++p)
       for (int i = g.first[p]; i < g.first[p] + g.count[p]; ++i) {
         const long long bs = p == 0 ? 0 : N + (long long)(p - 1) * N * k, q0 = bs + (long long)i * (p == 0 ? fa::kRows : g.qr);
-        tiles.push_back({p == 0 ? q0 + fa::kRows : (q0 - bs + g.qr) / k + (long long)fa::kKeys * p, (int)q0});
+        tiles[n++] = {p == 0 ? q0 + fa::kRows : (q0 - bs + g.qr) / k + (long long)fa::kKeys * p, (int)q0};
       }
-    std::stable_sort(tiles.begin(), tiles.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
-    for (int i = 0; i < g.n_qt; ++i) g.q0[i] = tiles[i].second;
+    std::sort(tiles, tiles + n,
+              [](const Tile& x, const Tile& y) { return x.keys != y.keys ? x.keys > y.keys : x.q0 < y.q0; });
+    for (int i = 0; i < n; ++i) g.q0[i] = tiles[i].q0;
   }
   const long long items = (long long)g.n_qt * H * B;
   const bool fits = items <= (1ll << 30);

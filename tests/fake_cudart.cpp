@@ -38,11 +38,14 @@ struct Call {
 cudaError_t launch(const void* f, dim3 g, dim3 b, size_t smem, int cluster, bool pdl) {
   if (g_launches_left == 0) return cudaErrorInvalidValue;
   if (g_launches_left > 0) --g_launches_left;
+  const bool fails = g_heap_fails;
+  g_heap_fails = false;              // (for this log's own allocations)
   const auto it = names().find(f);
   char line[512];
   snprintf(line, sizeof line, "%s|%u,%u,%u|%u|%zu|%d|%d\n", it == names().end() ? "?" : it->second.c_str(), g.x, g.y,
            g.z, b.x, smem, cluster, pdl ? 1 : 0);
   log() += line;
+  g_heap_fails = fails;
   return cudaSuccess;
 }
 CUresult encode_tiled(...) { return CUDA_SUCCESS; }

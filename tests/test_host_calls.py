@@ -1,5 +1,7 @@
 """Host code of the entry points, without a GPU (host_calls.py)."""
 import ctypes
+import subprocess
+import sys
 
 import pytest
 
@@ -113,3 +115,15 @@ def test_prefill_chunks(lib, monkeypatch, asked, lens, chunks):
     got = [x.grid[0] for x in launches(lib) if "embed_tokens" in x.kernel]
     dec.close()
     assert got == chunks
+
+
+@pytest.mark.parametrize("blocks,N,k", [(1, 1024, 4), (2, 301, 3), (2, 6000, 5)])     # listed tiles, and past the list
+def test_train_attention_without_heap(lib, blocks, N, k):
+    """No allocation, so no exception, between the C caller and the launch."""
+    T = N * (1 + blocks * k)
+    code = (f"import ctypes; lib = ctypes.CDLL({lib._name!r}); f = lib.kf_op_train_attention\n"
+            "f.argtypes = [ctypes.c_int32] * 7 + [ctypes.c_void_p] * 4 + [ctypes.c_int32, ctypes.c_void_p]\n"
+            f"call = lambda: f({blocks}, 1, 4, {N}, {k}, 0, {T}, {P}, {P}, {P}, {P}, 0, None)\n"
+            "call(); lib.fake_heap_fails(1); rc = call(); lib.fake_heap_fails(0); print('rc', rc)")
+    p = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
+    assert p.returncode == 0 and "rc 0" in p.stdout, p.stderr
