@@ -289,8 +289,8 @@ __global__ void __launch_bounds__(kThr, 3) k_train_attention(TrainAttnArgs a) {
 // The same attention on the 5th-generation tensor cores (k_attn_tc): an item is
 // up to 128 query rows of one (sequence, head), all of the context or of one
 // block.  A block's tiles hold whole windows (floor(128 / k) k rows, anchored
-// at the block's start), so that their keys in each block fit one 128-key
-// tile; tiles cut at 128 rows opened up to two tiles per block, and a tile
+// at the block's start) where those nearly fill it, so that their keys in each block
+// fit one 128-key tile; tiles cut at 128 rows opened up to two tiles per block, and a tile
 // across two parts of the layout the ranges of both.
 namespace {
 constexpr int kTileList = 448;
@@ -425,7 +425,13 @@ extern "C" int kf_op_train_attention(int32_t blocks, int32_t B, int32_t H, int32
   TrainArgs g{};
   g.a = a;
   g.n_batch = B;
-  g.qr = k <= fa::kRows ? fa::kRows / k * k : fa::kRows;
+  // Whole windows where they fill seven eighths of a tile, else 128 rows: a tile of
+  // few rows walks the context as a full one does (12 heads, N = 512, SingleForward,
+  // whole windows -> 128 rows, against the one-CTA kernel's time: k = 65 1.34 -> 0.69,
+  // k = 43 1.03 -> 0.69, k = 26 0.86 -> 0.70; filled tiles are the better ones at short
+  // contexts, N = 24: k = 29 0.80 -> 0.94, k = 9 0.85 -> 0.85)
+  const int whole = k <= fa::kRows ? fa::kRows / k * k : 0;
+  g.qr = 8 * whole >= 7 * fa::kRows ? whole : fa::kRows;
   for (int p = 0; p <= blocks; ++p) {
     const long long bs = p == 0 ? 0 : N + (long long)(p - 1) * N * k, len = p == 0 ? N : (long long)N * k;
     const long long lo = std::max<long long>(q_begin, bs) - bs, hi = std::min<long long>(q_end, bs + len) - bs;

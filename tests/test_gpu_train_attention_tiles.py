@@ -27,6 +27,8 @@ def _reference(torch, q, kk, v, mask):
     (2, 1, 2, 257, 5, None, None),     # 125-row tiles, two blocks
     (2, 1, 1, 3, 130, None, None),     # windows longer than a tile
     (1, 1, 1, 2, 128, None, None),     # a window is a tile
+    (1, 1, 2, 40, 43, None, None),     # 128-row tiles that cut windows of 43
+    (2, 1, 1, 30, 65, 31, 1950),       # ... and of 65, from a window's second row to its end
     (2, 1, 1, 200, 7, 13, 2777),       # a range that starts and ends inside tiles
     (2, 1, 2, 90, 4, 91, 449),         # rows of block 1 only, from the middle of a window
     (1, 1, 1, 300, 2, 299, 301),       # the last context row and the first noise row

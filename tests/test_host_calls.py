@@ -127,3 +127,14 @@ def test_train_attention_without_heap(lib, blocks, N, k):
             "call(); lib.fake_heap_fails(1); rc = call(); lib.fake_heap_fails(0); print('rc', rc)")
     p = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
     assert p.returncode == 0 and "rc 0" in p.stdout, p.stderr
+
+
+@pytest.mark.parametrize("k,rows", [(1, 128), (3, 126), (5, 125), (8, 128), (22, 128), (37, 128), (16, 128), (28, 112),
+                                    (43, 128), (65, 128), (100, 128), (112, 112), (127, 127), (128, 128), (200, 128)])
+def test_train_attention_query_tiles(lib, k, rows):
+    """A block's query tiles hold whole windows where those fill seven eighths of
+    128 rows, else 128 rows."""
+    N = 20
+    assert lib.kf_op_train_attention(1, 1, 1, N, k, 0, N * (1 + k), P, P, P, P, 0, None) == 0
+    (got,) = launches(lib)
+    assert got.grid[0] == 1 + -(-N * k // rows)
