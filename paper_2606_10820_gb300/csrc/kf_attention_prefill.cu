@@ -41,8 +41,9 @@ struct PrefillPolicy {
     r.cmin = im.pos0;
     fa::count_tiles(r);
   }
+  static __device__ __forceinline__ bool has_row(const Args&, const Item& im, int row) { return row < im.rows; }
   static __device__ __forceinline__ fa::RowVis vis(const Args&, const Item& im, int row) {
-    return {row < im.rows ? im.pos0 + row : -1, 0, 0, 0, 0};
+    return {im.pos0 + min(row, im.rows - 1), 0, 0, 0, 0};
   }
   static __device__ __forceinline__ void load_q(const Maps&, const Item&, uint32_t, uint32_t) {}
   // 32 rows of Q to bf16, swizzled as the MMA reads them (rows past the item: zeros)

@@ -115,7 +115,11 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 //   tile(a, it, kt, kend, lane, d_err)   what a key tile copies: TileRef, by warp 0's lanes
 //   tile_bytes / load_k / load_v   the bytes of a K (or V) tile and its copies
 //   clear_v(ref, lane, dst)   the V rows that no copy of this tile writes become zeros
-//   vis(a, it, row)      the row's visible keys (ctx = -1: no such row)
+//   has_row(a, it, row)  whether the item has this row
+//   vis(a, it, row)      the row's visible keys; a row that the item does not have is
+//                        given those of a row that it has (its result is not stored):
+//                        a row without keys would cost its warp the separate maximum
+//                        and the masks in every tile
 //   store(a, it, row, o, inv)   the finished row
 template <class P>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -319,7 +323,7 @@ k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args 
       for (int j = 0; j < r.n; ++j, ++g) {
         int kt, kend;
         tile_at(r, j, &kt, &kend);
-        const bool open = P::all_open(a) && kt + kKeys <= kend && kt + kKeys - 1 <= r.cmin && v.ctx >= 0;
+        const bool open = P::all_open(a) && kt + kKeys <= kend && kt + kKeys - 1 <= r.cmin;
         const bool masked = __any_sync(0xffffffffu, !open);
         // the keys of chunk c that this row sees (each key belongs to one
         // range's tiles)
@@ -465,7 +469,7 @@ k_attn_tc(const __grid_constant__ typename P::Maps maps, const typename P::Args 
         arrive(o_free);
         // every row of the item is written: one whose scores are NaN as NaN, not left
         // as the buffer was (a row with finite scores has l > 0)
-        if (v.ctx >= 0) P::store(a, im, row, o, 1.f / l);
+        if (P::has_row(a, im, row)) P::store(a, im, row, o, 1.f / l);
       }
     }
   }

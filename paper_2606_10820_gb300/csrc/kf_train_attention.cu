@@ -358,8 +358,11 @@ struct TrainPolicy {
     }
     fa::count_tiles(r);
   }
+  static __device__ __forceinline__ bool has_row(const Args& g, const Item& im, int row) {
+    return im.q0 + row >= g.a.q_begin && im.q0 + row < im.q1;
+  }
   static __device__ __forceinline__ RowVis vis(const Args& g, const Item& im, int row) {
-    return im.q0 + row < im.q1 ? row_vis(g.a, im.q0 + row) : RowVis{-1, 0, 0, 0, 0};
+    return row_vis(g.a, max(g.a.q_begin, min(im.q0 + row, im.q1 - 1)));
   }
   static __device__ __forceinline__ void load_q(const Maps& m, const Item& im, uint32_t dst, uint32_t bar) {
     tma_load_4d(dst, &m.q, bar, 0, im.h, im.q0, im.b);
