@@ -389,6 +389,406 @@ struct TrainPolicy {
 };
 }  // namespace
 
+// ------------------------------------------------------ tcgen05, few items
+// The same items with one CTA per SM, for calls whose items do not outnumber the
+// SMs: no second CTA is there to hide a chain's waits, so the chain itself is
+// shorter.  Two buffers each of S and P (S of tile g + 1 is computed while the
+// softmax works on tile g), and two threads per query row, each with half of its
+// keys and of its output (four measured 5 % slower):
+//   warp 0      TMA: an item's Q, then its K and V tiles into a four-stage ring;
+//   warp 1      S_g = Q K_g^T into one of two TMEM buffers, O += P_g V_g with P from
+//               shared memory (an item's last P V right after its last S);
+//   warps 2..9  the softmax: mask S_g, share the row maximum with the partner warp
+//               (the other half of the same rows), keep a reference per row that is
+//               raised when a tile's maximum exceeds it by more than 2^8, and write P_g
+//               as bf16 into shared memory (K-major, swizzled).
+// Tiles are numbered across the CTA's items (g).  Every wait is bounded; a wait
+// that runs out sets the error word and ends the CTA's loops.
+namespace {
+constexpr int kTcRows = 128;
+constexpr int kTcKeys = 128;
+constexpr int kTcSplit = 2;                          // softmax threads per query row
+constexpr int kTcSoftmax = 128 * kTcSplit;           // kTcSplit warps per TMEM lane quarter
+constexpr int kTcThreads = 64 + kTcSoftmax;
+constexpr int kTcPart = kTcKeys / kTcSplit;          // keys of a row per softmax thread
+constexpr int kTcOut = kHD / kTcSplit;               // output dims of a row per softmax thread
+constexpr uint32_t kTcTile = kTcRows * kHD * 2;       // 16 KB: Q, a K tile, a V tile
+constexpr uint32_t kTcP = kTcRows * kTcKeys * 2;      // 32 KB: one P tile (two 64-key atoms)
+// K/V ring stages: tile j's copies are issued while tile j - 1 is in the
+// softmax and tile j - 2's V still feeds P V (two stages measured 2.0 us per
+// tile, the copy latency on the critical path)
+constexpr int kTcStages = 4;
+// [Q][K stages][V stages][P 2], the barriers and shared scalars (256 B),
+// then the row-max exchange [2 tiles][kTcSplit parts][128 rows] and the row
+// sums [2 items][kTcSplit][128]
+constexpr size_t tc_smem_bytes() {
+  return 1024 + (1 + 2 * kTcStages) * (size_t)kTcTile + 2 * (size_t)kTcP + 256 + 4 * kTcSplit * 128 * 4;
+}
+
+// The two softmax warps of a TMEM lane quarter hold the two parts of the same
+// rows; they meet on named barrier 2 + quarter (64 threads), which also ORs
+// a predicate over them: both get the same answer and leave a loop together.
+__device__ __forceinline__ bool pair_bar_or(int quarter, bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, %2, 64, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)pred), "r"(2 + quarter)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void pair_bar(int quarter) {
+  asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kTcThreads, 1)
+k_train_attention_few(const __grid_constant__ TrainPolicy::Maps maps, const TrainArgs ga, int* d_err) {
+  extern __shared__ __align__(1024) uint8_t tsm_raw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tsm_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t sQ = smem_u32(sm);
+  const uint32_t sK = sQ + kTcTile;                  // [kTcStages]
+  const uint32_t sV = sK + kTcStages * kTcTile;      // [kTcStages]
+  constexpr uint32_t kPOff = (1 + 2 * kTcStages) * kTcTile;
+  uint8_t* Pp = sm + kPOff;                          // [2][2 atoms][128 rows][128 B]
+  const uint32_t sP = smem_u32(Pp);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kPOff + 2 * kTcP);
+  uint64_t* q_full = bars;
+  uint64_t* q_empty = bars + 1;                      // the item's last S product done
+  uint64_t* kv_full = bars + 2;                      // [kTcStages]
+  uint64_t* kv_empty = kv_full + kTcStages;          // [kTcStages]
+  uint64_t* s_full = kv_empty + kTcStages;           // [2]
+  uint64_t* p_full = s_full + 2;                     // [2]: P_g written (and S_g read)
+  uint64_t* o_full = p_full + 2;                     // [2]
+  uint64_t* o_free = o_full + 2;                     // the item's O read out
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 1);
+  int* s_cnt = reinterpret_cast<int*>(tmem_slot + 1);    // K/V tiles the MMA thread has taken
+  int* s_qcnt = s_cnt + 1;                               // Q tiles the MMA thread has taken
+  float* s_mx = reinterpret_cast<float*>(sm + kPOff + 2 * kTcP + 256);         // [2][kTcSplit][128]
+  float* s_l = s_mx + 2 * kTcSplit * kTcRows;                                  // [2][kTcSplit][128]
+
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int quarter = warp & 3;                 // softmax warps: TMEM lanes 32 quarter ..
+  const int row = 32 * quarter + lane;          // this softmax thread's query row in the tile
+  const int part = (warp - 2) >> 2;             // its keys kTcPart part .. and output dims kTcOut part ..
+  // (the word is set below, or after a wait of about 2 s)
+  if (t == 0 && blockIdx.x == 0) atomicExch(d_err, 0);
+  const int n_items = TrainPolicy::n_items(ga);
+  // the CTA's i-th item: rounds of gridDim.x items, walked forwards in even
+  // rounds and backwards in odd ones, so that each CTA's items add up to
+  // about the same number of tiles; -1 past the last
+  auto item_at = [&](int i) -> int {
+    const int P = gridDim.x, c = blockIdx.x;
+    const long long w = (long long)i * P + ((i & 1) ? P - 1 - c : c);
+    return w < n_items ? (int)w : -1;
+  };
+  if (t == 0) {
+    mbar_init(smem_u32(q_full), 1);
+    mbar_init(smem_u32(q_empty), 1);
+    for (int i = 0; i < kTcStages; ++i) {
+      mbar_init(smem_u32(&kv_full[i]), 1);
+      mbar_init(smem_u32(&kv_empty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&s_full[i]), 1);
+      mbar_init(smem_u32(&p_full[i]), kTcSoftmax);      // every softmax thread
+      mbar_init(smem_u32(&o_full[i]), 1);
+    }
+    mbar_init(smem_u32(o_free), kTcSoftmax);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.q)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.k)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.v)) : "memory");
+    s_cnt[0] = 0;
+    s_qcnt[0] = 0;
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+
+  if (warp == 0) {
+    bool ok = true;
+    int g = 0, issued = 0, q_issued = 0, it = 0;
+    for (int w = item_at(0); ok && w >= 0; w = item_at(++it)) {
+      TrainPolicy::Item im;
+      fa::Ranges r;
+      TrainPolicy::item(ga, w, lane, im, r);
+      if (lane == 0) {
+        // the Q buffer is free once the previous item's last S product is done
+        if (it > 0 && !mbar_wait(smem_u32(q_empty), (it - 1) & 1, d_err)) ok = false;
+        if (ok) {
+          mbar_expect_tx(smem_u32(q_full), kTcTile);
+          TrainPolicy::load_q(maps, im, sQ, smem_u32(q_full));
+          q_issued = it + 1;
+        }
+        for (int j = 0; ok && j < r.n; ++j, ++g) {
+          const int st = g % kTcStages;
+          if (g >= kTcStages && !mbar_wait(smem_u32(&kv_empty[st]), ((g / kTcStages) - 1) & 1, d_err)) {
+            ok = false;
+            break;
+          }
+          int kt, kend;
+          fa::tile_at(r, j, &kt, &kend);
+          mbar_expect_tx(smem_u32(&kv_full[st]), 2 * kTcTile);
+          tma_load_4d(sK + st * kTcTile, &maps.k, smem_u32(&kv_full[st]), 0, im.h, kt, im.b);
+          tma_load_4d(sV + st * kTcTile, &maps.v, smem_u32(&kv_full[st]), 0, im.h, kt, im.b);
+          issued = g + 1;
+        }
+      }
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+    }
+    if (lane == 0 && !ok) {
+      // let the copies still in flight land before the CTA ends (bounded)
+      for (int j = *(volatile int*)s_cnt; j < issued; ++j)
+        mbar_wait(smem_u32(&kv_full[j % kTcStages]), (j / kTcStages) & 1, d_err);
+      if (q_issued > *(volatile int*)s_qcnt) mbar_wait(smem_u32(q_full), (q_issued - 1) & 1, d_err);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    constexpr uint32_t idesc_s = idesc_bf16(kTcRows, kTcKeys);
+    constexpr uint32_t idesc_o = idesc_bf16(kTcRows, kHD) | (1u << 16);   // B (V) MN-major
+    bool ok = true;
+    int g = 0, it = 0, o_items = 0;
+    int pv = -1;                  // the tile whose S is issued and whose P V is not
+    bool pv_first = false;        // ... the first tile of its item
+    // O += P_i V_i in TMEM columns 256 .. 319.  An item's first tile
+    // overwrites O once the softmax has read the previous item's O out; the
+    // softmax rescales O in place before it releases P_i when the row max
+    // has grown.
+    auto issue_pv = [&](int i, bool first) -> bool {
+      if (first) {
+        if (o_items > 0 && !mbar_wait(smem_u32(o_free), (o_items - 1) & 1, d_err)) return false;
+        ++o_items;
+      }
+      const int st = i & 1;
+      if (!mbar_wait(smem_u32(&p_full[st]), (i >> 1) & 1, d_err)) return false;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int kvs = i % kTcStages;
+      const uint32_t pa = sP + st * kTcP, vb = sV + kvs * kTcTile;
+#pragma unroll
+      for (int kk = 0; kk < kTcKeys / 16; ++kk)
+        mma_bf16(tmem + 256, sdesc(pa + (kk >> 2) * (kTcP / 2) + (kk & 3) * 32),
+                 sdesc_mn(vb + kk * 16 * 128), idesc_o, (!first || kk > 0) ? 1u : 0u);
+      mma_commit(smem_u32(&o_full[st]));
+      mma_commit(smem_u32(&kv_empty[kvs]));
+      return true;
+    };
+    for (int w = item_at(0); ok && w >= 0; w = item_at(++it)) {
+      TrainPolicy::Item im;
+      fa::Ranges r;
+      TrainPolicy::item(ga, w, lane, im, r);
+      if (lane == 0) {
+        ok = mbar_wait(smem_u32(q_full), it & 1, d_err);
+        if (ok) *(volatile int*)s_qcnt = it + 1;
+        for (int j = 0; ok && j < r.n; ++j, ++g) {
+          const int st = g & 1;
+          if (!mbar_wait(smem_u32(&kv_full[g % kTcStages]), (g / kTcStages) & 1, d_err)) { ok = false; break; }
+          *(volatile int*)s_cnt = g + 1;
+          // S buffer st is free once the softmax has read S_{g-2}
+          if (g >= 2 && !mbar_wait(smem_u32(&p_full[st]), ((g - 2) >> 1) & 1, d_err)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t kb = sK + (g % kTcStages) * kTcTile;
+#pragma unroll
+          for (int kk = 0; kk < kHD / 16; ++kk)
+            mma_bf16(tmem + kTcKeys * st, sdesc(sQ + kk * 32), sdesc(kb + kk * 32), idesc_s, kk > 0 ? 1u : 0u);
+          mma_commit(smem_u32(&s_full[st]));
+          if (j == r.n - 1) mma_commit(smem_u32(q_empty));
+          if (pv >= 0 && !issue_pv(pv, pv_first)) { ok = false; break; }
+          pv = g;
+          pv_first = j == 0;
+          // the item's last P V follows at once: the softmax's read of O
+          // does not wait for the next item's copies
+          if (j == r.n - 1) {
+            if (!issue_pv(pv, pv_first)) { ok = false; break; }
+            pv = -1;
+          }
+        }
+        if (ok && r.n == 0) mma_commit(smem_u32(q_empty));
+      }
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+    }
+    if (lane == 0 && ok && pv >= 0) issue_pv(pv, pv_first);
+    __syncwarp();
+  } else {
+    // softmax: kTcSplit threads per query row, `part` of its keys and output each
+    static_assert(kTcPart % 32 == 0 && kTcPart <= 64 && (kTcOut == 16 || kTcOut == 32),
+                  "32-column TMEM loads of S, one load of O per thread");
+    const float sc = 1.4426950408889634f * rsqrtf((float)kHD);
+    const uint32_t lane_base = (uint32_t)(32 * quarter) << 16;
+    const int kb0 = kTcPart * part;               // first key of this thread's part of a tile
+    constexpr float kRescale = 8.f;
+    // this row's 16-byte chunks of P buffer 0 for keys kb0 .. kb0 + 31: atom
+    // kb0 / 64, chunks (kb0 % 64) / 8 + q at position chunk ^ (row % 8)
+    const uint32_t prow = sP + (kb0 >> 6) * (kTcP / 2) + row * 128;
+    const int chunk0 = (kb0 & 63) >> 3;
+    // this thread's output dims of the O accumulator in TMEM
+    const uint32_t o_addr = tmem + lane_base + 256 + kTcOut * part;
+    // A bounded wait that runs out marks the thread failed; the next
+    // OR-barrier tells its partner warp, and both leave the loops (the other
+    // pairs' waits then run out in turn).
+    bool failed = false;
+    auto wait_or_abort = [&](uint64_t* bar, uint32_t parity) {
+      if (!mbar_wait(smem_u32(bar), parity, d_err)) failed = true;
+    };
+    bool ok = true;
+    int g = 0, it = 0;
+    for (int w = item_at(0); ok && w >= 0; w = item_at(++it)) {
+      TrainPolicy::Item im;
+      fa::Ranges r;
+      TrainPolicy::item(ga, w, lane, im, r);
+      const RowVis v = TrainPolicy::vis(ga, im, row);
+      // the visible keys kb0 + i (i < kTcPart) of a row as a bit mask: [lo, hi) relative to the tile
+      auto range_bits = [&](int lo, int hi) -> unsigned long long {
+        lo = max(lo - kb0, 0);
+        hi = min(hi - kb0, kTcPart);
+        if (hi <= lo) return 0ull;
+        const unsigned long long up = hi >= 64 ? ~0ull : ((1ull << hi) - 1ull);
+        return up & ~((1ull << lo) - 1ull);
+      };
+      // m: the row max the probabilities of the item's tiles so far are
+      // taken against (raised only when a tile's max exceeds it by more than
+      // 2^8, so P stays below 256); l: this thread's part of their sum
+      float m = -INFINITY, l = 0.f;
+      for (int j = 0; j < r.n; ++j, ++g) {
+        const int st = g & 1;
+        int kt, kend;
+        fa::tile_at(r, j, &kt, &kend);
+        // visible keys of this part: the context prefix [0, ctx], the windows,
+        // none past the range's end (each key belongs to one range's tiles)
+        const int lim = min(kend - kt, kTcKeys);
+        const bool open = !ga.a.dense && kt + kTcKeys - 1 < kend && kt + kTcKeys - 1 <= r.cmin;
+        unsigned long long vis = ~0ull;
+        if (!open)
+          vis = (range_bits(0, v.ctx - kt + 1) | range_bits(v.w1lo - kt, v.w1hi - kt) |
+                 range_bits(v.w2lo - kt, v.w2hi - kt)) &
+                range_bits(0, lim);
+        wait_or_abort(&s_full[st], (g >> 1) & 1);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        float sv[kTcPart];
+#pragma unroll
+        for (int c = 0; c < kTcPart / 32; ++c) tmem_ld32(tmem + lane_base + kTcKeys * st + kb0 + 32 * c, sv + 32 * c);
+        // raw scores: sc > 0, so the max commutes with the scaling
+        if (vis != ~0ull) {
+#pragma unroll
+          for (int e = 0; e < kTcPart; ++e) sv[e] = ((vis >> e) & 1ull) ? sv[e] : -INFINITY;
+        }
+        // four independent max chains, then combined
+        float mq[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int e = 0; e < kTcPart; e += 8)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) mq[c] = max3f(mq[c], sv[e + 2 * c], sv[e + 2 * c + 1]);
+        float mx = fmaxf(fmaxf(mq[0], mq[1]), fmaxf(mq[2], mq[3]));
+        // the row's max over its parts (the partner warp)
+        s_mx[(st * kTcSplit + part) * kTcRows + row] = mx;
+        if (pair_bar_or(quarter, failed)) { ok = false; break; }
+        mx = s_mx[(st * kTcSplit) * kTcRows + row];
+#pragma unroll
+        for (int q = 1; q < kTcSplit; ++q) mx = fmaxf(mx, s_mx[(st * kTcSplit + q) * kTcRows + row]);
+        // A new reference max when this tile's exceeds it by more than 2^8: O
+        // and l so far are scaled to it (O once the previous tile's P V has
+        // landed; nothing is accumulated before a finite max).  The TMEM
+        // load and store are warp-wide: a warp rescales when any of its rows
+        // needs it, the others by 1.
+        const bool raise = mx * sc > m + kRescale;
+        const float f = (raise && m != -INFINITY) ? ex2(m - mx * sc) : 1.f;
+        if (__any_sync(0xffffffffu, f != 1.f)) {
+          wait_or_abort(&o_full[(g - 1) & 1], ((g - 1) >> 1) & 1);
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          float rr[kTcOut];
+          tmem_ld32(o_addr, rr);
+#pragma unroll
+          for (int d = 0; d < kTcOut; ++d) rr[d] *= f;
+          tmem_st32(o_addr, rr);
+        }
+        if (raise) {
+          l *= f;
+          m = mx * sc;
+        }
+        const float mn = m;
+        // P = exp2(S sc - mn) rounded to bf16 (ex2(-inf) = 0 for masked keys),
+        // the sum of the rounded values
+        const uint32_t pbase = prow + st * kTcP;
+        const float nmn = mn == -INFINITY ? 0.f : -mn;
+        const uint64_t sc2 = f2(sc, sc), nmn2 = f2(nmn, nmn);
+        uint64_t ps2[4] = {f2(0.f, 0.f), f2(0.f, 0.f), f2(0.f, 0.f), f2(0.f, 0.f)};   // independent sums
+#pragma unroll
+        for (int q = 0; q < kTcPart / 8; ++q) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int e = 8 * q + 2 * u;
+            const float2 arg = f2_split(fma_f2(f2(sv[e], sv[e + 1]), sc2, nmn2));
+            pk[u] = pack_bf16(ex2(arg.x), ex2(arg.y));
+            const float2 pf = unpack_bf16(pk[u]);
+            ps2[u] = add_f2(ps2[u], f2(pf.x, pf.y));
+          }
+          const uint32_t addr = pbase + (((chunk0 + q) ^ (row & 7)) << 4);
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(pk[0]), "r"(pk[1]), "r"(pk[2]),
+                       "r"(pk[3])
+                       : "memory");
+        }
+        const float2 ps = f2_split(add_f2(add_f2(ps2[0], ps2[1]), add_f2(ps2[2], ps2[3])));
+        l += ps.x + ps.y;
+        // S_g read, P_g written: to the tensor cores (async proxy); every
+        // softmax thread arrives
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&p_full[st])) : "memory");
+      }
+      if (!ok) break;
+      float o[kTcOut];
+#pragma unroll
+      for (int d = 0; d < kTcOut; ++d) o[d] = 0.f;
+      if (r.n > 0) {
+        // the item's last P V completes the accumulator; once every softmax
+        // thread has read it, the next item's first P V may overwrite it
+        wait_or_abort(&o_full[(g - 1) & 1], ((g - 1) >> 1) & 1);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tmem_ld32(o_addr, o);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        if (pair_bar_or(quarter, failed)) { ok = false; break; }
+        asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(o_free)) : "memory");
+      }
+      // the row's sum over its parts, in a fixed order (one buffer per item
+      // parity: a thread writes the next item's sums only after the pair
+      // barrier below, which its partner passes after reading this item's)
+      float* sl = s_l + (it & 1) * kTcSplit * kTcRows;
+      sl[part * kTcRows + row] = l;
+      pair_bar(quarter);
+      float lt = 0.f;
+#pragma unroll
+      for (int q = 0; q < kTcSplit; ++q) lt += sl[q * kTcRows + row];
+      if (TrainPolicy::has_row(ga, im, row)) {
+        const TrainAttnArgs& a = ga.a;
+        const float inv = 1.f / lt;
+        float* dst = a.out + (((size_t)im.b * (a.q_end - a.q_begin) + (im.q0 + row - a.q_begin)) * a.H + im.h) * kHD +
+                     kTcOut * part;
+#pragma unroll
+        for (int d = 0; d < kTcOut; d += 4)
+          *reinterpret_cast<float4*>(dst + d) = make_float4(o[d] * inv, o[d + 1] * inv, o[d + 2] * inv, o[d + 3] * inv);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
 }  // namespace kf
 
 using namespace kf;
@@ -444,6 +844,7 @@ extern "C" int kf_op_train_attention(int32_t blocks, int32_t B, int32_t H, int32
     g.count[p] = (int)((hi + rows - 1) / rows) - g.first[p];
     g.n_qt += g.count[p];
   }
+  long long longest = a.dense ? T : 0;     // keys of the longest listed tile
   if (g.n_qt <= kTileList) {
     // sorted by the context keys a tile's last row sees (the windows add about
     // the same to every block tile), then by position; on the stack: nothing
@@ -459,17 +860,32 @@ extern "C" int kf_op_train_attention(int32_t blocks, int32_t B, int32_t H, int32
     std::sort(tiles, tiles + n,
               [](const Tile& x, const Tile& y) { return x.keys != y.keys ? x.keys > y.keys : x.q0 < y.q0; });
     for (int i = 0; i < n; ++i) g.q0[i] = tiles[i].q0;
+    longest = std::max(longest, tiles[0].keys);
   }
   const long long items = (long long)g.n_qt * H * B;
   const bool fits = items <= (1ll << 30);
   int* err = op_error_word(s, !fits);   // cleared by the kernel, if it runs
   if (!err) return KF_E_CUDA;
   if (!fits) return KF_E_ARG;
-  static PerDevice attr_tc;
-  set_smem_attr(attr_tc, fa::k_attn_tc<TrainPolicy>, fa::kSmemBytes);
-  // persistent: two CTAs per SM over the (query tile, head, sequence) items
-  const dim3 grid((unsigned)std::min<long long>(items, 2ll * device_sms()));
-  kf_launch(fa::k_attn_tc<TrainPolicy>, grid, dim3(fa::kThreads), fa::kSmemBytes, s, maps, g, err, 1);
+  // One CTA per SM while that gives every SM an item at most, and with long chains
+  // (1024 keys and more) up to two; past that two CTAs per SM, which hide each
+  // other's waits.  One CTA -> two, microseconds: 2 heads, N = 1024, k = 4 (80 items)
+  // 15.4 / 18.8; 8 heads, N = 1024, k = 2 (192) 15.5 / 20.1; 6 heads, N = 2048,
+  // k = 1 (192) 24.4 / 31.9; 12 heads, N = 1024, k = 2 (288) 20.4 / 21.7; but 12
+  // heads, N = 384, k = 4 (180) 14.2 / 13.2, 8 heads, N = 1024, k = 4 (320) 25.1 / 21.1
+  const int num_sms = device_sms();
+  if (items <= num_sms || (items <= 2 * num_sms && longest >= 1024)) {
+    static PerDevice attr_few;
+    set_smem_attr(attr_few, k_train_attention_few, tc_smem_bytes());
+    const dim3 grid((unsigned)std::min<long long>(items, num_sms));
+    kf_launch(k_train_attention_few, grid, dim3(kTcThreads), tc_smem_bytes(), s, maps, g, err);
+  } else {
+    // persistent: two CTAs per SM over the (query tile, head, sequence) items
+    static PerDevice attr_tc;
+    set_smem_attr(attr_tc, fa::k_attn_tc<TrainPolicy>, fa::kSmemBytes);
+    const dim3 grid((unsigned)std::min<long long>(items, 2ll * num_sms));
+    kf_launch(fa::k_attn_tc<TrainPolicy>, grid, dim3(fa::kThreads), fa::kSmemBytes, s, maps, g, err, 1);
+  }
   if (cudaGetLastError() == cudaSuccess) return KF_OK;
   op_error_word(s);
   return KF_E_CUDA;

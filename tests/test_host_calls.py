@@ -138,3 +138,17 @@ def test_train_attention_query_tiles(lib, k, rows):
     assert lib.kf_op_train_attention(1, 1, 1, N, k, 0, N * (1 + k), P, P, P, P, 0, None) == 0
     (got,) = launches(lib)
     assert got.grid[0] == 1 + -(-N * k // rows)
+
+
+@pytest.mark.parametrize("blocks,H,N,k,few", [
+    (1, 1, 32, 1, True), (2, 3, 384, 8, False), (1, 8, 384, 5, True),    # 2, 153 and 152 items
+    (1, 8, 1024, 2, True), (1, 8, 1024, 4, False),                       # 192 and 320 of up to 1,024 keys
+    (1, 24, 512, 2, False), (1, 48, 1024, 4, False),
+])
+def test_train_attention_kernel(lib, blocks, H, N, k, few):
+    """One CTA per SM while the items do not outnumber the SMs (long ones: twice
+    the SMs), two past that."""
+    assert lib.kf_op_train_attention(blocks, 1, H, N, k, 0, N * (1 + blocks * k), P, P, P, P, 0, None) == 0
+    (got,) = launches(lib)
+    assert ("train_attention_few" in got.kernel) == few
+    assert got.grid[0] <= (152 if few else 304)
