@@ -4,8 +4,9 @@ whole fp32 decode steps against the oracle (needs a GB300).
 The row counts B (P + k) cover one row, the 16-row groups and their
 remainders, 64 rows and several 64-row tiles; d = 160 and d_ff = 192 leave a
 short last K stage and a ragged last column tile; noise_hidden = 2112 splits
-K over a cluster.  The oracle runs in fp64: with |logit| below 2 and sums of
-at most 2,112 fp32 products over a few layers, 1e-4 is about 50 fp32 roundings.
+K over a cluster.  The oracle runs in fp64.  Largest |logit| differences seen:
+2.4e-7 after AR steps, 1.0e-5 after steps with noise (the fp32 angles
+noise_scale * z of the noise features); the bounds are four times those.
 """
 import numpy as np
 import pytest
@@ -51,6 +52,6 @@ def test_fp32_steps_at_tile_edges(kf, batch, ks):
         got = dec.step(k, z)
         lg = dec.logits(max(k, 1))
         want, rl = ref.step(k, z, want_logits=True)
-        assert np.abs(lg - rl).max() < 1e-4
+        assert np.abs(lg - rl).max() < (4e-5 if k else 1e-6)
         assert np.array_equal(got, want.astype(np.int32))
     dec.close()

@@ -152,3 +152,36 @@ def test_train_attention_kernel(lib, blocks, H, N, k, few):
     (got,) = launches(lib)
     assert ("train_attention_few" in got.kernel) == few
     assert got.grid[0] <= (152 if few else 304)
+
+
+def _names(lib):
+    return [x.kernel for x in launches(lib)]
+
+
+def test_pair_tests_run_pairs(lib, monkeypatch):
+    """The shapes of test_gpu_pair_gemm.py reach the kernels they are there for."""
+    import numpy as np
+    import test_gpu_pair_gemm as tp
+    from paper_2606_10820_gb300 import kforcing as kf
+    from synth import MEDIUM, OWT, make_prompts, make_weights
+    for shapes, kernel in ((tp.PAIR_PRODUCTS, "k_gemm_tc_pair<256, 6, 6>"), (tp.LOOP_PRODUCTS, "k_gemm_tc_persist<256")):
+        for shape in shapes:
+            assert lib.kf_op_gemm_bf16(GEMM_TC, *shape, P, P, P, None) == 0
+            assert kernel in _names(lib)[0], shape
+    assert _head(lib, *tp.HEAD_ON_PAIRS) == 0
+    assert "k_gemm_tc_pair<256, 6, 4>" in _names(lib)[0]
+    monkeypatch.setattr(kf, "_lib", lib)
+    cfg = OWT.replace(n_layer=1, vocab=67)
+    dec = kf.Decoder(cfg, make_weights(cfg), max_batch=16, max_k=1)
+    lib.fake_clear()
+    dec.prefill(make_prompts(tp.MLP_UP_LENS, cfg.vocab))
+    assert any("k_gemm_tc_pair<256, 6, 1>" in n for n in _names(lib))      # bias + GELU
+    dec.close()
+    cfg = MEDIUM.replace(n_layer=1, vocab=tp.LOGITS_V, max_len=32)
+    dec = kf.Decoder(cfg, make_weights(cfg), max_batch=37, max_k=4, flags=kf.KF_FLAG_NO_GRAPH)
+    dec.prefill(make_prompts([4] * 37, cfg.vocab))
+    dec.step(4, np.zeros((37, 4), np.float32))
+    lib.fake_clear()
+    dec.logits(4)
+    assert any("k_gemm_tc_pair<256, 4, 5>" in n for n in _names(lib))      # logits
+    dec.close()
