@@ -68,16 +68,6 @@ __device__ __forceinline__ void clear_error(const TcArgs& g) {
   if (g.clear_err && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) atomicExch(g.d_err, 0);
 }
 
-// Nothing of a CTA's may be under way when it ends: its copies of the last
-// `issued` stages have landed.  They have unless a wait ran out and the MMA thread
-// stopped; then each wait here is bounded too, and the first that runs out is the
-// last (a copy that takes two seconds does not come)
-template <int STAGES>
-__device__ __forceinline__ void drain_copies(const uint64_t* full, uint32_t issued, int* d_err) {
-  for (uint32_t i = issued - min(issued, (uint32_t)STAGES); i < issued; ++i)
-    if (!mbar_wait(smem_u32(&full[i % STAGES]), (i / STAGES) & 1, d_err)) return;
-}
-
 __device__ __forceinline__ void epi_bar() {
   asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
 }
@@ -415,8 +405,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
       }
       pdl_wait();
       for (int i = 0; i < pre; ++i) issue(i, smem_u32(smem + i * STAGE_BYTES), smem_u32(&bars[i]), false);
-      int i = pre;
-      for (; i < nst; ++i) {
+      for (int i = pre; i < nst; ++i) {
         const int s = i % STAGES;
         const uint32_t ph = (i / STAGES) & 1;
         if (!mbar_wait(smem_u32(&bars[STAGES + s]), ph ^ 1, g.d_err)) break;
@@ -426,7 +415,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
         issue(i, sa, full, true);
         issue(i, sa, full, false);
       }
-      if (pw == 0) drain_copies<STAGES>(bars, i, g.d_err);
     }
     __syncwarp();
   }
@@ -691,7 +679,7 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     // predecessor kernel finishes.
     if (lane == 0) {
       const bool wp = warp != 0;
-      uint32_t stage = 0, issued = 0;
+      uint32_t stage = 0;
       bool first = true;
       for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
         const int m0 = tile_m0(t), n0 = tile_n0(t);
@@ -708,7 +696,6 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
               tma_load_2d(smem_u32(smem + i * STAGE_BYTES), &map_a, smem_u32(&full[i]), i * kBK, m0);
           }
           i0 = pre;
-          issued = pre;
           first = false;
         }
         bool live = true;
@@ -726,12 +713,10 @@ k_gemm_tc_persist(const __grid_constant__ CUtensorMap map_a, const __grid_consta
           } else {
             tma_load_2d(sa + A_ATOM, &map_w, fb, i * kBK, n0);
           }
-          issued = sc + 1;
         }
         if (!live) break;
         stage += nkb;
       }
-      if (!wp) drain_copies<STAGES>(full, issued, g.d_err);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -853,6 +838,19 @@ __device__ __forceinline__ void st_row_bf16(__nv_bfloat16* p, const float* v) {
   }
 }
 
+// After a wait that ran out: the copies of the last stages, of `issued` in all, are
+// waited for on the leader, whose barriers count both CTAs' copies, and the peer
+// waits for the leader at the end: no CTA of the pair ends with copies under way to
+// its shared memory or its barriers.  These waits are bounded too, and the first
+// that runs out is the last (a copy that takes two seconds does not come).  The
+// leader's producer does so for its own stages, the thread whose wait for the
+// accumulator ran out for all of the pair's, which the producers may have issued
+// without another wait.  When nothing ran out every copy has been consumed
+__device__ __forceinline__ void drain_copies(const uint64_t* full, uint32_t stages, uint32_t issued, int* d_err) {
+  for (uint32_t i = issued - min(issued, stages); i < issued; ++i)
+    if (!mbar_wait(smem_u32(&full[i % stages]), (i / stages) & 1, d_err)) return;
+}
+
 template <int BN, int STAGES, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w, TcArgs g) {
@@ -910,7 +908,7 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
   if (warp == 0) {
     if (lane == 0) {
-      uint32_t stage = 0, issued = 0;
+      uint32_t stage = 0;
       bool first = true, live = true;
       for (int t = pair; live && t < tiles; t += pairs) {
         const int m0 = tile_m0(t), n0 = tile_n0(t) + (int)rank * (BN / 2);
@@ -928,12 +926,12 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           for (int i = 0; i < pre; ++i)
             tma_load_2d_pair(smem_u32(smem + i * STAGE_BYTES), &map_a, map_rank(smem_u32(&full[i]), 0), i * kBK, m0);
           i0 = pre;
-          issued = pre;
           first = false;
         }
         for (int i = i0; i < nkb; ++i) {
           const uint32_t sc = stage + i, s = sc % STAGES;
           if (!mbar_wait_cluster(smem_u32(&empty[s]), ((sc / STAGES) & 1) ^ 1, g.d_err)) {
+            if (rank == 0) drain_copies(full, STAGES, sc, g.d_err);   // (both CTAs' copies)
             live = false;
             break;
           }
@@ -942,15 +940,9 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           if (rank == 0) mbar_expect_tx(smem_u32(&full[s]), 2 * STAGE_BYTES);
           tma_load_2d_pair(sa, &map_a, fb, i * kBK, m0);
           tma_load_2d_pair(sa + A_ATOM, &map_w, fb, i * kBK, n0);
-          issued = sc + 1;
         }
         stage += nkb;
       }
-      // the last products' arrivals on this CTA's barriers, and on the leader, whose
-      // barriers count both CTAs' copies, these (the peer waits for it below)
-      for (uint32_t i = issued - min(issued, (uint32_t)STAGES); i < issued; ++i)
-        if (!mbar_wait_cluster(smem_u32(&empty[i % STAGES]), (i / STAGES) & 1, g.d_err)) break;
-      if (rank == 0) drain_copies<STAGES>(full, issued, g.d_err);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -993,7 +985,11 @@ k_gemm_tc_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       float rinv = 1.f;                           // while the mainloop runs
       if (EPI == EPI_BIAS_GELU && g.epi.ss_in) rinv = in ? row_rinv(g.epi, row) : 0.f;
       const bool ok = mbar_wait_cluster(smem_u32(&accf[buf]), (ti >> 1) & 1, g.d_err);
-      if (!__all_sync(0xffffffffu, ok)) break;    // timed out: the leader stops too
+      if (!__all_sync(0xffffffffu, ok)) {         // timed out: the leader stops too
+        if (rank == 0 && warp == 2 && lane == 0)
+          drain_copies(full, STAGES, ceil_div(tiles - pair, pairs) * nkb, g.d_err);
+        break;
+      }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t acc = tmem + buf * BN + ((uint32_t)(quarter * 32) << 16);
       if (EPI == EPI_HEAD) {
