@@ -705,10 +705,11 @@ int kf_init(const kf_config* cfg_in, const kf_weights* w, void* stream, kf_ctx**
 // The rows of a chunk's attention groups: 128 (tcgen05) once the 128-row items
 // cover the SMs and hold 40 rows or more on average, else 16 (warp-level MMA, which
 // also splits the keys of few long rows).  Measured, 768-wide model, 4 layers,
-// 16-row -> 128-row groups, microseconds per prefill: 16 prompts of 128-896
-// 1334 -> 1196, 64 of 64 530 -> 487, 64 of 48 441 -> 424, 4 of 400 (192 items) 355
-// -> 344; but 64 of 32 364 -> 368, 64 of 17 284 -> 300, 16 of 32 221 -> 235, one of
-// 1000 (96 items) 312 -> 344, 4 of 128 (48 items) 218 -> 239.
+// 16-row -> 128-row groups, microseconds per prefill with an AR step and its
+// logits: 16 prompts of 128-896 1225 -> 1060, 64 of 64 782 -> 752, 64 of 48 710 ->
+// 697, 64 of 40 587 -> 571, 4 of 400 (192 items) 482 -> 466; but 64 of 32 641 -> 646,
+// 64 of 17 467 -> 470, 16 of 32 387 -> 391, one of 1000 (96 items) 432 -> 438, 4 of
+// 128 (48 items) 352 -> 363.
 static int prefill_group_rows(const kf_ctx* c, const std::vector<int4>& runs) {
   if (!c->bf16 || c->hd != 64) return kMaxGroupRows;
   long long rows = 0, tiles = 0;

@@ -11,8 +11,8 @@
 //   warps 2..5  the softmax, one thread per query row (its TMEM lane), so the
 //            maximum and the sum need no exchange between threads; P goes back to
 //            TMEM, not through shared memory.
-// Two CTAs share an SM (113 KB of shared memory, 256 TMEM columns and 168 registers a
-// thread each): while one's chain of MMA, TMEM loads and exponentials waits, the
+// Two CTAs share an SM (113 KB of shared memory, 256 TMEM columns and 150 of at most
+// 168 registers a thread each): while one's chain of MMA, TMEM loads and exponentials waits, the
 // other's runs.  The scores are taken against a reference per row that is fixed by
 // the first tile the row sees keys in and stays while no later score exceeds it by
 // 2^8, so a tile is one pass over its scores, and S is released before the last
@@ -23,8 +23,8 @@
 // against 93, 95 and 125) but lets O overflow from |V| near 2^63 / keys.  32-key chunks that no row of a warp sees (a window tile's
 // other windows, a prefix tile past the diagonal) are zeros in P and nothing else.
 // Measured (training attention, 4 x 12 heads, N = 1024, k = 4, SingleForward; and 3 x
-// 7 heads, N = 301, k = 3, DoubleForward): 129 -> 94 us (343 TFLOP/s over the mask's
-// pairs) and 45 -> 26 us, against one CTA per SM with two threads per row, P through
+// 7 heads, N = 301, k = 3, DoubleForward): 131 -> 94 us (343 TFLOP/s over the mask's
+// pairs) and 45 -> 22.8 us, against one CTA per SM with two threads per row, P through
 // shared memory and a maximum exchanged per tile.  A tile takes an SM about 2,700
 // clocks: 512 of exponentials, 700 of MMA, about 950 issue slots per scheduler; the
 // rest is latency (TMEM loads, barriers, instruction fetch) that two chains do not

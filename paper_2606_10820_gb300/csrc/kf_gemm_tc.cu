@@ -1339,10 +1339,14 @@ int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   // microseconds.  Row epilogues, from three rounds: MLP-up 4096 x 3072 x 768 in
   // a step 28.4 -> 26.0, 4096 x 4096 x 1024 37.3 -> 35.4; fp32 products 4096 x
   // 3072 x 768 26.5 -> 24.7, 4096 x 4096 x 1024 39.0 -> 32.8, 8192 x 4096 x 4096
-  // 190 -> 153 (1.80 PFLOP/s); at two rounds 2560 x 3072 x 768 15.8 -> 16.9.
+  // 190 -> 153 (1.80 PFLOP/s); at two rounds 2560 x 3072 x 768 15.8 -> 16.9.  Below
+  // K = 768 the start weighs too much, however many the rounds: 8192 x 16,384 (27
+  // rounds) at K = 640 161 -> 162, 512 138 -> 156, 256 101 -> 145; 4096 x 3072 at
+  // K = 640 20.0 -> 22.2 (8192 x 4096 gains at 640 yet, 45.4 -> 42.4).
   // Records and logits: 2048 x 50,257 at K = 1024 162 -> 146, K = 768 147 -> 134,
   // 1024 x 50,257 x 768 (11 rounds) 74.3 -> 71.5, 512 x 50,257 x 1024 (6) 57.3 ->
-  // 52.7; but 1024 x 30,522 x 768 (7) 47.6 -> 51.5, 2100 x 50,257 x 256 82 -> 99;
+  // 52.7; but 1024 x 30,522 x 768 (7) 47.6 -> 51.5, 2100 x 50,257 x 256 82 -> 99 (the
+  // line is coarse at small K: 2048 x 50,257 x 512, deep, 88 -> 94);
   // logits 2048 x 50,257 197 -> 179.  Not with one or three row tiles, where half or a
   // quarter of the pairs' CTAs have no rows (LM head and selection, greedy: 1 row x
   // 50,257 x 2048 48 -> 64, 1 x 131,072 x 1024 56 -> 80, 300 x 131,072 x 512 57 -> 68,
@@ -1418,7 +1422,7 @@ int launch_gemm_tc(const GemmDesc& g, int* d_err, cudaStream_t s) {
   if (ceil_div(g.N, 256) * m_tiles <= num_sms && ceil_div(g.N, 192) * m_tiles <= num_sms &&
       ceil_div(g.N, 192) > ceil_div(g.N, 256))
     return launch_bn<192, 5, 1>(g, d_err, num_sms, s);
-  if (g.epi.kind != EPI_HEAD && persist && ceil_div(g.N, 256) * m_tiles > num_sms)
+  if (persist && ceil_div(g.N, 256) * m_tiles > num_sms)
     return launch_persist<256, 3>(g, d_err, num_sms, s);
   return launch_bn<256, 4, 1>(g, d_err, num_sms, s);
 }

@@ -119,8 +119,9 @@ enum EpiKind : int {
 
 struct HeadRec {   // one record per (head row, chunk of 32 vocab ids)
   float m;         // max of l over the chunk
-  float s;         // sum over the chunk of exp(l - m), ascending id order
-  int a;           // lowest id attaining m
+  float s;         // sum over the chunk of exp(l - m): in ascending id order (FP32-FMA
+                   // kernel) or in four packed partial sums (tcgen05 kernels)
+  int a;           // lowest id attaining m (without want_arg: the chunk's first id)
   int pad;
 };
 
